@@ -738,7 +738,10 @@ emt_status run_loop(emt_ctx* c, int32_t max_iterations, emt_run_stats* st)
         }
         int side = (int)(c->it & 1), cin = (int)(c->it % 3), cout = (int)((c->it + 1) % 3),
             cclr = (int)((c->it + 2) % 3);
-        int64_t chunks = (c->live_g + c->block - 1) / c->block + (c->live_c + c->block - 1) / c->block;
+        // the fused step takes block-sized chunks, the transport kernel
+        // warp-sized ones (a block for every warp chunk while blocks last)
+        const int per = c->plan.split && c->opt.max_active <= 0 ? 32 : c->block;
+        int64_t chunks = (c->live_g + per - 1) / per + (c->live_c + per - 1) / per;
         int grid = (int)std::max<int64_t>(1, std::min<int64_t>(chunks, c->resident_blocks));
         EMT_CUDA(c, cudaEventRecord(c->ev0, c->stream));
         cudaError_t e =

@@ -49,59 +49,72 @@ constexpr int transport_threads_per_sm()
 template <int G, bool X, typename R>
 __device__ __forceinline__ void transport_lane(const Params<R>& p, const Tracks<R>& qo, Counters* co,
                                                const InterQueue<R>& iq, int* n_iq, bool count_queued, int lane,
-                                               TrackReg<R>& t, bool active, bool held, long long src, unsigned* eh)
+                                               TrackReg<R>& t, bool active, bool held, long long src, unsigned* eh,
+                                               StepTally& tally)
 {
     const unsigned lanes_below = (1u << lane) - 1u;
     Effects fx;
     StepOut<R> o;
     o.n = 0;
     int model = kNoInteraction;
-    int substeps = 0;
+    int live = 1;
+    bool finish = false;
     if (held) {
         copy_out(t, o);
     } else if (active) {
         bool alive;
         model = transport_part<G, X>(p, t, fx, alive);
-        substeps = fx.substeps;
-        if (model == kNoInteraction) {
-            finish_step(p, t, alive, fx, o);
-            apply_effects(p, t.ev, t.type, t.step, fx);
-        }
+        tally.substeps += (unsigned)fx.substeps;
+        finish = model == kNoInteraction;
+        if (finish) finish_step(p, t, alive, fx, o);
     }
-    count_substeps(p, lane, substeps);
-    {
-        const unsigned ms = __ballot_sync(0xFFFFFFFFu, active && !held && (count_queued || model == kNoInteraction));
-        if (lane == 0 && ms) atomicAdd(&p.total_steps[0], (unsigned long long)__popc(ms));
-    }
-    emit<1>(p, qo, co, lane, o, t.x, t.ev, t.vol, eh);
-    // queue the interacting tracks
+    tally.steps += __popc(__ballot_sync(0xFFFFFFFFu, active && !held && (count_queued || model == kNoInteraction)));
+    // the output and queue reservations and the live counts all wait for the
+    // L2 (about 740 clocks each): issued together, used below
     const bool need = model != kNoInteraction;
-    const unsigned m = __ballot_sync(0xFFFFFFFFu, need);
-    if (m) {
-        int base = 0;
-        if (lane == 0) base = atomicAdd(n_iq, __popc(m));
-        base = __shfl_sync(0xFFFFFFFFu, base, 0);
-        if (need) {
-            const long long k = (long long)base + __popc(m & lanes_below);
-            if (k < p.Q) {
-                iq.x[k] = t.x[0];
-                iq.y[k] = t.x[1];
-                iq.z[k] = t.x[2];
-                iq.ux[k] = t.u[0];
-                iq.uy[k] = t.u[1];
-                iq.uz[k] = t.u[2];
-                iq.T[k] = t.T;
-                iq.uid[k] = t.uid;
-                iq.dep[k] = fx.dep;
-                iq.ev[k] = t.ev;
-                iq.step[k] = t.step;
-                iq.tv[k] = pack_tvm(t.type, t.vol, model);
-                iq.src[k] = (uint32_t)src;
-            } else {
-                atomicOr(p.status, kStatusQueueOverflow);
-            }
+    const unsigned mg = __ballot_sync(0xFFFFFFFFu, o.n > 0 && o.type[0] == 0);
+    const unsigned mc = __ballot_sync(0xFFFFFFFFu, o.n > 0 && o.type[0] != 0);
+    const unsigned mi = __ballot_sync(0xFFFFFFFFu, need);
+    unsigned long long base = 0;
+    int qbase = 0;
+    if (lane == 0) {
+        if (mg | mc) base = reserve_outputs(co, __popc(mg), __popc(mc));
+        if (mi) qbase = atomicAdd(n_iq, __popc(mi));
+    }
+    if (finish) live = apply_effects(p, t.ev, t.type, t.step, fx);
+    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    qbase = __shfl_sync(0xFFFFFFFFu, qbase, 0);
+    if (o.n > 0) {
+        const long long dst = o.type[0] == 0 ? (long long)(uint32_t)base + __popc(mg & lanes_below)
+                                             : p.Q - 1 - ((long long)(uint32_t)(base >> 32) + __popc(mc & lanes_below));
+        if (dst < 0 || dst >= p.Q) {
+            atomicOr(p.status, kStatusQueueOverflow);
+        } else {
+            store_track(qo, dst, t.x, o.u[0], o.T[0], o.uid[0], t.ev, o.step[0], o.type[0], t.vol);
+            if (eh) atomicAdd(&eh[energy_class(est_f(o.T[0]))], 1u);
         }
     }
+    if (need) {
+        const long long k = (long long)qbase + __popc(mi & lanes_below);
+        if (k < p.Q) {
+            iq.x[k] = t.x[0];
+            iq.y[k] = t.x[1];
+            iq.z[k] = t.x[2];
+            iq.ux[k] = t.u[0];
+            iq.uy[k] = t.u[1];
+            iq.uz[k] = t.u[2];
+            iq.T[k] = t.T;
+            iq.uid[k] = t.uid;
+            iq.dep[k] = fx.dep;
+            iq.ev[k] = t.ev;
+            iq.step[k] = t.step;
+            iq.tv[k] = pack_tvm(t.type, t.vol, model);
+            iq.src[k] = (uint32_t)src;
+        } else {
+            atomicOr(p.status, kStatusQueueOverflow);
+        }
+    }
+    report_finished(p, t.ev, live);
 }
 
 // The charged tracks of a step in a field, sorted by expected cost (a
@@ -184,7 +197,7 @@ __global__ void __launch_bounds__(BS, transport_threads_per_sm<R>() / BS)
     __shared__ unsigned s_eh[S ? kEBins : 1];
     __shared__ Selection s_sel, s_spill;
     constexpr bool select = S;
-    if (blockIdx.x == 0 && threadIdx.x == 0) p.cnt[cclr] = Counters{};
+    if (blockIdx.x == 0) clear_counters(&p.cnt[cclr]);
     const Tracks<R> qi = p.q[side];
     const Tracks<R> qo = p.q[side ^ 1];
     const int nG = p.cnt[cin].n[0];
@@ -207,11 +220,16 @@ __global__ void __launch_bounds__(BS, transport_threads_per_sm<R>() / BS)
         const int chunksG = (nG + 31) >> 5;
         const int chunksC = (nC + 31) >> 5;
         const bool sorted = p.has_field != 0;
-        for (;;) {
-            int chunk = 0;
-            if (lane == 0) chunk = atomicAdd(&p.cnt[cin].work, 1);
-            chunk = __shfl_sync(0xFFFFFFFFu, chunk, 0);
-            if (chunk >= chunksG + chunksC) break;
+        StepTally tally;
+        // The first chunk of a warp is fixed: warp 0 of every block before
+        // warp 1 of any, so that the first (in a field: the most expensive)
+        // chunks run on different SMs.  Later chunks come from the
+        // dispenser, whose answer is on its way during the current chunk.
+        const int warps = (int)gridDim.x * (BS / 32);
+        int chunk = (int)blockIdx.x + (int)gridDim.x * (tid >> 5);
+        while (chunk < chunksG + chunksC) {
+            int next = 0;
+            if (lane == 0) next = warps + atomicAdd(&p.cnt[cin].work, 1);
             const bool photon_chunk = charged_first ? chunk >= chunksC : chunk < chunksG;
             const int local = photon_chunk ? (charged_first ? chunk - chunksC : chunk)
                                            : (charged_first ? chunk : chunk - chunksG);
@@ -221,8 +239,11 @@ __global__ void __launch_bounds__(BS, transport_threads_per_sm<R>() / BS)
             const long long src = photon_chunk ? i : Q - nC + i;
             TrackReg<R> t;
             if (active) load_track(qi, src, t);
-            transport_lane<G, X>(p, qo, co, p.iq, &p.cnt[cin].n_int, true, lane, t, active, false, src, nullptr);
+            transport_lane<G, X>(p, qo, co, p.iq, &p.cnt[cin].n_int, true, lane, t, active, false, src, nullptr,
+                                 tally);
+            chunk = __shfl_sync(0xFFFFFFFFu, next, 0);
         }
+        flush_tally(p, lane, tally);
         return;
     }
 
@@ -250,6 +271,7 @@ __global__ void __launch_bounds__(BS, transport_threads_per_sm<R>() / BS)
     }
     const int chunksG = (nG + BS - 1) / BS;
     const int chunksC = (nC + BS - 1) / BS;
+    StepTally tally;
     for (;;) {
         if (tid == 0) s_chunk = atomicAdd(&p.cnt[cin].work, 1);
         __syncthreads();
@@ -313,8 +335,9 @@ __global__ void __launch_bounds__(BS, transport_threads_per_sm<R>() / BS)
             const unsigned mh = __ballot_sync(0xFFFFFFFFu, held);
             if (lane == 0 && mh) atomicAdd(&p.total_steps[2], (unsigned long long)__popc(mh));
         }
-        transport_lane<G, X>(p, qo, co, p.iq, &p.cnt[cin].n_int, true, lane, t, active, held, src, s_eh);
+        transport_lane<G, X>(p, qo, co, p.iq, &p.cnt[cin].n_int, true, lane, t, active, held, src, s_eh, tally);
     }
+    flush_tally(p, lane, tally);
     if constexpr (select) {
         __syncthreads();
         for (int b = threadIdx.x; b < kEBins; b += BS)
@@ -362,19 +385,21 @@ __device__ __forceinline__ void interact_chunks(const Params<R>& p, const Tracks
                                                 Counters* co, int cin, const InterQueue<R>& iq, int n_int,
                                                 long long spare, bool unlimited, const InterQueue<R>& qnext,
                                                 int* n_next, unsigned* eh, int& s_chunk, int* count, int* offset,
-                                                unsigned short* perm)
+                                                unsigned short* perm, StepTally& tally)
 {
     constexpr int CH = BS * kInteractRecords;
     const int chunks = (n_int + CH - 1) / CH;
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const unsigned lanes_below = (1u << lane) - 1u;
-    for (;;) {
-        if (tid == 0) s_chunk = atomicAdd(&p.cnt[cin].work_b, 1);
+    // the first chunk by block number, later ones from the dispenser, whose
+    // answer is on its way while the current chunk is sampled
+    int chunk = blockIdx.x;
+    while (chunk < chunks) {
+        int next = 0;
+        if (tid == 0) next = (int)gridDim.x + atomicAdd(&p.cnt[cin].work_b, 1);
         if (tid < kNumModels) count[tid] = 0;
         __syncthreads();
-        const int chunk = s_chunk;
-        if (chunk >= chunks) break;
         const long long r0 = (long long)chunk * CH;
         const int n_here = (int)(n_int - r0 < CH ? n_int - r0 : CH);
         // counting sort of the chunk's records by model
@@ -465,36 +490,34 @@ __device__ __forceinline__ void interact_chunks(const Params<R>& p, const Tracks
                     }
                 }
             }
-            if (stepped) apply_effects(p, t.ev, t.type, t.step, fx);
-            {
-                const unsigned md = __ballot_sync(0xFFFFFFFFu, mine && !stepped);
-                if constexpr (kPipe) {
-                    // the step of an interacting track counts when it commits
-                    const unsigned mc = __ballot_sync(0xFFFFFFFFu, mine && stepped);
-                    if (lane == 0 && mc) atomicAdd(&p.total_steps[0], (unsigned long long)__popc(mc));
-                    if (lane == 0 && md) atomicAdd(&p.total_steps[1], (unsigned long long)__popc(md));
-                    if (md) {
-                        int base = 0;
-                        if (lane == 0) base = atomicAdd(n_next, __popc(md));
-                        base = __shfl_sync(0xFFFFFFFFu, base, 0);
-                        if (mine && !stepped) {
-                            const long long k = (long long)base + __popc(md & lanes_below);
-                            if (k < p.Q)
-                                copy_record(iq, r, qnext, k);
-                            else
-                                atomicOr(p.status, kStatusQueueOverflow);
-                        }
-                    }
-                } else {
-                    if (lane == 0 && md) {
-                        atomicAdd(&p.total_steps[0], -(unsigned long long)__popc(md));
-                        atomicAdd(&p.total_steps[1], (unsigned long long)__popc(md));
+            int live = 1;
+            if (stepped) live = apply_effects(p, t.ev, t.type, t.step, fx);
+            const unsigned md = __ballot_sync(0xFFFFFFFFu, mine && !stepped);
+            tally.deferred += __popc(md);
+            if constexpr (kPipe) {
+                // the step of an interacting track counts when it commits
+                tally.steps += __popc(__ballot_sync(0xFFFFFFFFu, mine && stepped));
+                if (md) {
+                    int base = 0;
+                    if (lane == 0) base = atomicAdd(n_next, __popc(md));
+                    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+                    if (mine && !stepped) {
+                        const long long k = (long long)base + __popc(md & lanes_below);
+                        if (k < p.Q)
+                            copy_record(iq, r, qnext, k);
+                        else
+                            atomicOr(p.status, kStatusQueueOverflow);
                     }
                 }
+            } else {
+                tally.steps -= __popc(md);
             }
             emit<2>(p, qo, co, lane, o, t.x, t.ev, t.vol, eh);
+            report_finished(p, t.ev, live);
         }
+        if (tid == 0) s_chunk = next;
         __syncthreads();
+        chunk = s_chunk;
     }
 }
 
@@ -513,9 +536,11 @@ __global__ void __launch_bounds__(BS, 512 / BS) k_interact(Params<R> p, int side
         __syncthreads();
     }
     const long long ntot = (long long)p.cnt[cin].n[0] + p.cnt[cin].n[1];
+    StepTally tally;
     interact_chunks<R, BS, X, false>(p, p.q[side], p.q[side ^ 1], &p.cnt[cout], cin, p.iq, p.cnt[cin].n_int,
                                      p.Q - ntot, 2 * ntot <= p.Q, p.iq, nullptr, select ? s_eh : nullptr, s_chunk,
-                                     count, offset, perm);
+                                     count, offset, perm, tally);
+    flush_tally(p, threadIdx.x & 31, tally);
     if constexpr (select) {
         for (int b = threadIdx.x; b < kEBins; b += BS)
             if (s_eh[b]) atomicAdd(&p.ehist[(size_t)cout * kEBins + b], s_eh[b]);
@@ -553,7 +578,7 @@ __global__ void __launch_bounds__(BS, pipe_threads_per_sm<R>() / BS)
     __shared__ int count[kNumModels];
     __shared__ int offset[kNumModels + 1];
     __shared__ unsigned short perm[CH];
-    if (blockIdx.x == 0 && threadIdx.x == 0) p.cnt[cclr] = Counters{};
+    if (blockIdx.x == 0) clear_counters(&p.cnt[cclr]);
     const Tracks<R> qi = p.q[side];
     const Tracks<R> qo = p.q[side ^ 1];
     const InterQueue<R> q_prev = side ? p.iq : p.iq_alt;
@@ -567,8 +592,9 @@ __global__ void __launch_bounds__(BS, pipe_threads_per_sm<R>() / BS)
     Counters* const co = &p.cnt[cout];
 
     // interactions of the previous iteration
+    StepTally tally;
     interact_chunks<R, BS, X, true>(p, qi, qo, co, cin, q_prev, n_prev, Q - ntot, 2 * ntot <= Q, q_next, n_next,
-                                    nullptr, s_chunk, count, offset, perm);
+                                    nullptr, s_chunk, count, offset, perm, tally);
 
     // transport of this iteration's tracks (charged first in a field, in
     // the order of k_sort_order)
@@ -576,11 +602,16 @@ __global__ void __launch_bounds__(BS, pipe_threads_per_sm<R>() / BS)
     const int chunksG = (nG + 31) >> 5;
     const int chunksC = (nC + 31) >> 5;
     const bool charged_first = p.has_field != 0;
-    for (;;) {
-        int chunk = 0;
-        if (lane == 0) chunk = atomicAdd(&p.cnt[cin].work, 1);
-        chunk = __shfl_sync(0xFFFFFFFFu, chunk, 0);
-        if (chunk >= chunksG + chunksC) break;
+    // The first chunk of a warp is fixed, as in k_transport, starting with
+    // the blocks that had no interactions to sample.
+    const int grid = (int)gridDim.x;
+    const int busy = min((n_prev + CH - 1) / CH, grid);
+    const int warps = grid * (BS / 32);
+    int chunk = ((int)blockIdx.x < busy ? (int)blockIdx.x + grid - busy : (int)blockIdx.x - busy) +
+                grid * (int)(threadIdx.x >> 5);
+    while (chunk < chunksG + chunksC) {
+        int next = 0;
+        if (lane == 0) next = warps + atomicAdd(&p.cnt[cin].work, 1);
         const bool photon_chunk = charged_first ? chunk >= chunksC : chunk < chunksG;
         const int local = photon_chunk ? (charged_first ? chunk - chunksC : chunk)
                                        : (charged_first ? chunk : chunk - chunksG);
@@ -590,8 +621,10 @@ __global__ void __launch_bounds__(BS, pipe_threads_per_sm<R>() / BS)
         const long long src = photon_chunk ? i : Q - nC + i;
         TrackReg<R> t;
         if (active) load_track(qi, src, t);
-        transport_lane<G, X>(p, qo, co, q_next, n_next, false, lane, t, active, false, src, nullptr);
+        transport_lane<G, X>(p, qo, co, q_next, n_next, false, lane, t, active, false, src, nullptr, tally);
+        chunk = __shfl_sync(0xFFFFFFFFu, next, 0);
     }
+    flush_tally(p, lane, tally);
 }
 
 }  // namespace emt

@@ -111,27 +111,50 @@ __device__ __forceinline__ void finish_track(const Params<R>& p, uint32_t ev, in
 
 // An event is finished when its live-track count reaches zero.  A thread
 // adds its secondaries before removing its own track, so the count of an
-// event cannot touch zero while one of its tracks is still alive.
+// event cannot touch zero while one of its tracks is still alive.  The
+// returned atomic takes about 740 clocks: apply_effects issues it and
+// returns the count it leaves, report_finished looks at that once the step's
+// outputs are written.
 template <typename R>
-__device__ __forceinline__ void update_live(const Params<R>& p, uint32_t ev, int delta)
+__device__ __forceinline__ void report_finished(const Params<R>& p, uint32_t ev, int live)
 {
-    if (delta == 0) return;
-    int old = atomicAdd(&p.live[ev], delta);
-    if (old + delta == 0) {
-        unsigned k = atomicAdd(p.done_head, 1u);
-        p.done_ring[k % (unsigned)p.max_events] = ev;
-    }
+    if (live != 0) return;
+    const unsigned k = atomicAdd(p.done_head, 1u);
+    p.done_ring[k % (unsigned)p.max_events] = ev;
 }
 
+// the event's live-track count after the step (1, never "finished", when
+// the step did not change it)
 template <typename R>
-__device__ __forceinline__ void apply_effects(const Params<R>& p, uint32_t ev, int type, uint32_t steps,
-                                              const Effects& fx)
+__device__ __forceinline__ int apply_effects(const Params<R>& p, uint32_t ev, int type, uint32_t steps,
+                                             const Effects& fx)
 {
+    int live = 1;
+    if (fx.live_delta != 0) live = atomicAdd(&p.live[ev], fx.live_delta) + fx.live_delta;
     deposit_now(p, ev, fx.col, fx.dep);
     if (nonzero(fx.esc)) atomicAdd(&p.ledger[3 * (size_t)ev + 0], fx.esc);
     if (nonzero(fx.kill)) atomicAdd(&p.ledger[3 * (size_t)ev + 1], fx.kill);
     if (fx.finished) finish_track(p, ev, type, steps);
-    update_live(p, ev, fx.live_delta);
+    return live;
+}
+
+// Track-steps taken and deferred by a warp (the same in every lane) and RK4
+// evaluations of each lane, kept in registers and added to the run's totals
+// once per kernel.
+struct StepTally {
+    int steps = 0, deferred = 0;
+    unsigned substeps = 0;
+};
+
+// every lane of the warp calls it
+template <typename R>
+__device__ __forceinline__ void flush_tally(const Params<R>& p, int lane, const StepTally& c)
+{
+    const unsigned sub = p.has_field ? __reduce_add_sync(0xFFFFFFFFu, c.substeps) : 0u;
+    if (lane != 0) return;
+    if (c.steps) atomicAdd(&p.total_steps[0], (unsigned long long)(long long)c.steps);
+    if (c.deferred) atomicAdd(&p.total_steps[1], (unsigned long long)c.deferred);
+    if (sub) atomicAdd(&p.total_steps[3], (unsigned long long)sub);
 }
 
 // Phase A of one step of one track, in the order
@@ -504,16 +527,6 @@ __device__ __forceinline__ int field_substeps_estimate(const Params<R>& p, const
     return n < 1.0f ? 1 : (n > (float)kMaxSubsteps ? kMaxSubsteps : (int)n);
 }
 
-// RK4 evaluations of a warp's steps into the run's counter (field only;
-// every lane of the warp calls it)
-template <typename R>
-__device__ __forceinline__ void count_substeps(const Params<R>& p, int lane, int substeps)
-{
-    if (!p.has_field) return;
-    const unsigned v = __reduce_add_sync(0xFFFFFFFFu, (unsigned)substeps);
-    if (lane == 0 && v) atomicAdd(&p.total_steps[3], (unsigned long long)v);
-}
-
 template <typename R>
 __device__ __forceinline__ void load_track(const Tracks<R>& q, long long i, TrackReg<R>& t)
 {
@@ -562,8 +575,17 @@ __device__ __forceinline__ void copy_out(const TrackReg<R>& t, StepOut<R>& o)
     o.step[0] = t.step;
 }
 
+// Reserve ng photon and nc charged output slots with one atomic on the two
+// adjacent counts (neither count reaches 2^31, so no carry passes between
+// them); returns the first photon slot in the low word, charged in the high.
+__device__ __forceinline__ unsigned long long reserve_outputs(Counters* c, int ng, int nc)
+{
+    return atomicAdd(reinterpret_cast<unsigned long long*>(c->n),
+                     (unsigned long long)(uint32_t)ng | ((unsigned long long)(uint32_t)nc << 32));
+}
+
 // warp-aggregated reservation and store of each lane's outputs (all lanes
-// of the warp call it); counts are packed as photons | charged << 16.
+// of the warp call it).
 // With track selection on, eh (shared memory) counts the outputs' energy
 // classes.  kMaxOut: the most outputs a lane can have (1 after the
 // transport part, 2 after an interaction); the loops over the outputs are
@@ -573,47 +595,28 @@ __device__ __forceinline__ void emit(const Params<R>& p, const Tracks<R>& qo, Co
                                      const StepOut<R>& o, const double x[3], uint32_t ev, int vol,
                                      unsigned* eh = nullptr)
 {
+    unsigned mg[kMaxOut], mc[kMaxOut];
     int ng = 0, nc = 0;
 #pragma unroll
     for (int k = 0; k < kMaxOut; ++k) {
-        if (k < o.n) {
-            if (o.type[k] == 0)
-                ++ng;
-            else
-                ++nc;
-        }
+        mg[k] = __ballot_sync(0xFFFFFFFFu, k < o.n && o.type[k] == 0);
+        mc[k] = __ballot_sync(0xFFFFFFFFu, k < o.n && o.type[k] != 0);
+        ng += __popc(mg[k]);
+        nc += __popc(mc[k]);
     }
-    const int v = ng | (nc << 16);
-    int incl = v;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        int y = __shfl_up_sync(0xFFFFFFFFu, incl, off);
-        if (lane >= off) incl += y;
-    }
-    const int excl = incl - v;
-    const int tot = __shfl_sync(0xFFFFFFFFu, incl, 31);
-    if (tot == 0) return;
-    int baseG = 0, baseC = 0;
-    if (lane == 31) {
-        int tg = tot & 0xFFFF, tc = tot >> 16;
-        if (tg) baseG = atomicAdd(&cout->n[0], tg);
-        if (tc) baseC = atomicAdd(&cout->n[1], tc);
-    }
-    baseG = __shfl_sync(0xFFFFFFFFu, baseG, 31);
-    baseC = __shfl_sync(0xFFFFFFFFu, baseC, 31);
-    long long og = (long long)baseG + (excl & 0xFFFF);
-    long long oc = (long long)baseC + (excl >> 16);
+    if (ng + nc == 0) return;
+    unsigned long long base = 0;
+    if (lane == 0) base = reserve_outputs(cout, ng, nc);
+    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    const unsigned below = (1u << lane) - 1u;
+    long long og = (long long)(uint32_t)base, oc = (long long)(uint32_t)(base >> 32);
     const long long Q = p.Q;
 #pragma unroll
     for (int k = 0; k < kMaxOut; ++k) {
         if (k >= o.n) break;
-        long long dst;
-        if (o.type[k] == 0) {
-            dst = og++;
-        } else {
-            dst = Q - 1 - oc;
-            ++oc;
-        }
+        const long long dst = o.type[k] == 0 ? og + __popc(mg[k] & below) : Q - 1 - (oc + __popc(mc[k] & below));
+        og += __popc(mg[k]);
+        oc += __popc(mc[k]);
         if (dst < 0 || dst >= Q) {
             atomicOr(p.status, kStatusQueueOverflow);
             continue;
@@ -707,9 +710,7 @@ template <typename R, int BS, int G, bool X>
 __device__ __forceinline__ void step_body(const Params<R>& p, int side, int cin, int cout, int cclr, int& s_chunk,
                                           Staging<R, BS>& sg)
 {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        p.cnt[cclr] = Counters{};
-    }
+    if (blockIdx.x == 0) clear_counters(&p.cnt[cclr]);
     const Tracks<R> qi = p.q[side];
     const Tracks<R> qo = p.q[side ^ 1];
     const int nG = p.cnt[cin].n[0];
@@ -725,13 +726,16 @@ __device__ __forceinline__ void step_body(const Params<R>& p, int side, int cin,
     const int lane = tid & 31;
     const unsigned lanes_below = (1u << lane) - 1u;
     Counters* const co = &p.cnt[cout];
+    StepTally tally;
 
-    for (;;) {
-        if (tid == 0) s_chunk = atomicAdd(&p.cnt[cin].work, 1);
+    // the first chunk by block number, later ones from the dispenser, whose
+    // answer is on its way while the current chunk is stepped
+    int chunk = blockIdx.x;
+    while (chunk < chunksG + chunksC) {
+        int next = 0;
+        if (tid == 0) next = (int)gridDim.x + atomicAdd(&p.cnt[cin].work, 1);
         if (tid < kNumModels) sg.count[tid] = 0;
         __syncthreads();
-        const int chunk = s_chunk;
-        if (chunk >= chunksG + chunksC) break;
         const bool photon_chunk = chunk < chunksG;
         const long long i = photon_chunk ? (long long)chunk * bs + tid : (long long)(chunk - chunksG) * bs + tid;
         const long long n_here = photon_chunk ? nG : nC;
@@ -745,25 +749,22 @@ __device__ __forceinline__ void step_body(const Params<R>& p, int side, int cin,
         o.n = 0;
         int model = kNoInteraction;
         int rank = 0;
-        int substeps = 0;
+        int live = 1;
         if (active) {
             load_track(qi, src, t);
             bool alive;
             model = transport_part<G, X>(p, t, fx, alive);
-            substeps = fx.substeps;
+            tally.substeps += (unsigned)fx.substeps;
             if (model == kNoInteraction) {
                 finish_step(p, t, alive, fx, o);
-                apply_effects(p, t.ev, t.type, t.step, fx);
+                live = apply_effects(p, t.ev, t.type, t.step, fx);
             } else {
                 rank = atomicAdd(&sg.count[model], 1);
             }
         }
-        count_substeps(p, lane, substeps);
-        {
-            const unsigned ms = __ballot_sync(0xFFFFFFFFu, active);
-            if (lane == 0 && ms) atomicAdd(&p.total_steps[0], (unsigned long long)__popc(ms));
-        }
+        tally.steps += __popc(__ballot_sync(0xFFFFFFFFu, active));
         emit<1>(p, qo, co, lane, o, t.x, t.ev, t.vol);
+        report_finished(p, t.ev, live);
         __syncthreads();
         if (tid == 0) {
             int acc = 0;
@@ -844,17 +845,18 @@ __device__ __forceinline__ void step_body(const Params<R>& p, int side, int cin,
                 }
             }
         }
-        if (stepped) apply_effects(p, t.ev, t.type, t.step, fx);
-        {
-            const unsigned md = __ballot_sync(0xFFFFFFFFu, mine && !stepped);
-            if (lane == 0 && md) {
-                atomicAdd(&p.total_steps[0], -(unsigned long long)__popc(md));
-                atomicAdd(&p.total_steps[1], (unsigned long long)__popc(md));
-            }
-        }
+        live = 1;
+        if (stepped) live = apply_effects(p, t.ev, t.type, t.step, fx);
+        const int nd = __popc(__ballot_sync(0xFFFFFFFFu, mine && !stepped));
+        tally.steps -= nd;
+        tally.deferred += nd;
         emit<2>(p, qo, co, lane, o, t.x, t.ev, t.vol);
+        report_finished(p, t.ev, live);
+        if (tid == 0) s_chunk = next;
         __syncthreads();
+        chunk = s_chunk;
     }
+    flush_tally(p, lane, tally);
 }
 
 template <typename R, int BS, int G, bool X>
