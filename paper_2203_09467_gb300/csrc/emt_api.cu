@@ -213,6 +213,19 @@ const char* check_geometry(const emt_layer* layers, int n, const emt_world* w, i
     return nullptr;
 }
 
+// Ends of the energy grid and find_bin's guess: with the FP32 bits i of E,
+// i 2^-23 - 127 is log2 E less 0 to 0.087 (0.043 on average), and the
+// interval number is bpd log10(2) (log2 E - log2 grid[0]).
+template <typename R>
+void set_bin_guess(Params<R>& p, R lo, R hi, int bpd)
+{
+    p.grid_lo = lo;
+    p.grid_hi = hi;
+    const double per_octave = bpd * std::log10(2.0);
+    p.bin_scale = (float)(per_octave * 0x1p-23);
+    p.bin_offset = (float)(-per_octave * (127.0 - 0.043 + (lo > R(0) ? std::log2((double)lo) : 0.0)));
+}
+
 // geometry, field and scoring fields of the kernel parameters
 template <typename R>
 void set_geometry(Params<R>& p, int n, const emt_world* w)
@@ -1127,10 +1140,18 @@ emt_status emt_load_materials(emt_ctx* c, const emt_material* mats, int32_t n, c
     b.dgridf = c->mixed() ? c->at<float>(pl.dgridf) : nullptr;
     b.dtabf = c->mixed() ? c->at<float>(pl.dtabf) : nullptr;
     EMT_CUDA(c, build_tables(b, c->at<double>(pl.scratch), c->stream));
+    // the ends of the grid as the kernels see them (kernel parameters)
+    double ends[2] = {0.0, 0.0};
+    float endsf[2] = {0.f, 0.f};
+    for (int k = 0; k < 2; ++k) {
+        const size_t node = k ? (size_t)n_grid - 1 : 0;
+        EMT_CUDA(c, cudaMemcpyAsync(&ends[k], b.grid + node, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+        if (c->mixed())
+            EMT_CUDA(c, cudaMemcpyAsync(&endsf[k], b.gridf + node, sizeof(float), cudaMemcpyDeviceToHost, c->stream));
+    }
     EMT_CUDA(c, cudaStreamSynchronize(c->stream));
     c->n_mat = n;
     c->n_grid = n_grid;
-    float l10 = (float)std::log10(ph->grid_lo_MeV);
     for (int k = 0; k < 3; ++k) {
         c->pd.cut[k] = ph->cut_MeV[k];
         c->pf.cut[k] = ph->cut_MeV[k];
@@ -1149,8 +1170,8 @@ emt_status emt_load_materials(emt_ctx* c, const emt_material* mats, int32_t n, c
     c->pf.dgrid = c->at<float>(pl.dgridf);
     c->pf.dtab = c->at<float>(pl.dtabf);
     c->pd.n_grid = c->pf.n_grid = n_grid;
-    c->pd.bpd = c->pf.bpd = ph->bins_per_decade;
-    c->pd.log10_lo = c->pf.log10_lo = l10;
+    set_bin_guess(c->pd, ends[0], ends[1], ph->bins_per_decade);
+    set_bin_guess(c->pf, endsf[0], endsf[1], ph->bins_per_decade);
     c->pd.step_frac = c->pf.step_frac = ph->step_frac;
     c->pd.mask = c->pf.mask = ph->process_mask;
     c->pd.final_range = c->pf.final_range = ph->final_range_cm;
@@ -1688,7 +1709,13 @@ extern "C" emt_status emt_transport_static(int32_t device, uint32_t seed, const 
     b.dtab = reinterpret_cast<double*>(pool + pl.dtab);
     b.dgridf = nullptr;
     b.dtabf = nullptr;
-    if (build_tables(b, reinterpret_cast<double*>(pool + pl.scratch), st) != cudaSuccess) return EMT_ERR_CUDA;
+    double ends[2] = {0.0, 0.0};
+    if (build_tables(b, reinterpret_cast<double*>(pool + pl.scratch), st) != cudaSuccess ||
+        cudaMemcpyAsync(&ends[0], b.grid, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaMemcpyAsync(&ends[1], b.grid + n_grid - 1, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)
+        return EMT_ERR_CUDA;
+    set_bin_guess(p, ends[0], ends[1], ph->bins_per_decade);
     for (int k = 0; k < 3; ++k) {
         p.cut[k] = ph->cut_MeV[k];
         p.cutf[k] = (float)ph->cut_MeV[k];
@@ -1700,8 +1727,6 @@ extern "C" emt_status emt_transport_static(int32_t device, uint32_t seed, const 
     p.dgrid = b.dgrid;
     p.dtab = b.dtab;
     p.n_grid = n_grid;
-    p.bpd = ph->bins_per_decade;
-    p.log10_lo = (float)std::log10(ph->grid_lo_MeV);
     p.step_frac = ph->step_frac;
     p.final_range = ph->final_range_cm;
     p.mask = ph->process_mask;

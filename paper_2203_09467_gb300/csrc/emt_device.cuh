@@ -218,8 +218,8 @@ struct Params {
     const R* dgrid;  // grid[n+1] - grid[n]
     const R* dtab;   // layout of tab: tab[n+1][q] - tab[n][q]
     int n_grid;
-    int bpd;
-    float log10_lo;  // log10(grid[0]) for the bin guess
+    float bin_scale, bin_offset;  // bin guess from the FP32 bits of an energy (find_bin)
+    R grid_lo, grid_hi;           // grid[0], grid[n_grid - 1]
     const double* bk;
     const int* vacuum;
     const double* x0;     // radiation length per material (cm)
@@ -467,14 +467,16 @@ __host__ __device__ __forceinline__ long long ord_key(double a)
     return b < 0 ? -m : m;
 }
 
-// node n with grid[n] <= E < grid[n+1], clamped to [0, n_grid-2]: an FP32
-// logarithm guesses, exact comparisons with the nodes decide.
+// node n with grid[n] <= E < grid[n+1], clamped to [0, n_grid-2]: the FP32
+// bit pattern of E, read as a fixed-point number, is a piecewise-linear
+// log2 E (at most 0.087 below it), which guesses the interval within a
+// quarter of a bin at 8 bins per decade; exact comparisons with the nodes
+// decide.
 template <typename R>
 __device__ __forceinline__ int find_bin(const Params<R>& p, R E)
 {
-    float g = ((float)p.bpd) * (log10f(est_f(E)) - p.log10_lo);
-    int n = (int)g;
-    int top = p.n_grid - 2;
+    int n = (int)fmaf((float)__float_as_int(est_f(E)), p.bin_scale, p.bin_offset);
+    const int top = p.n_grid - 2;
     n = n < 0 ? 0 : (n > top ? top : n);
     while (n > 0 && !le_pos(p.grid[n], E)) --n;
     while (n < top && le_pos(p.grid[n + 1], E)) ++n;
@@ -494,13 +496,13 @@ __device__ __forceinline__ Lookup<R> locate_energy(const Params<R>& p, R E)
 {
     Lookup<R> l;
     l.clamp = 0;
-    if (le_pos(E, p.grid[0])) {
+    if (le_pos(E, p.grid_lo)) {
         l.clamp = -1;
         l.n = 0;
         l.f = R(0);
         return l;
     }
-    if (le_pos(p.grid[p.n_grid - 1], E)) {
+    if (le_pos(p.grid_hi, E)) {
         l.clamp = 1;
         l.n = p.n_grid - 2;
         l.f = R(0);
@@ -525,7 +527,7 @@ __device__ __forceinline__ R xs_value(const Params<R>& p, const R* t, const R* d
 template <typename R>
 __device__ __forceinline__ R range_value(const Params<R>& p, const R* t, const R* dt, R T, const Lookup<R>& l)
 {
-    if (lt_pos(T, p.grid[0])) return t[3] * mdiv(T, p.grid[0]);
+    if (lt_pos(T, p.grid_lo)) return t[3] * mdiv(T, p.grid_lo);
     int n = l.n;
     R f = l.f;
     if (l.clamp > 0) f = (T - p.grid[n]) * p.igrid[n];
@@ -538,7 +540,7 @@ __device__ __forceinline__ R range_value(const Params<R>& p, const R* t, const R
 template <typename R>
 __device__ __forceinline__ R inv_range(const Params<R>& p, const R* t, const R* irs, R r, int nstart)
 {
-    if (lt_pos(r, t[3])) return p.grid[0] * mdiv(r, t[3]);
+    if (lt_pos(r, t[3])) return p.grid_lo * mdiv(r, t[3]);
     int n = nstart;
     while (n > 0 && !le_pos(t[n * kNq + 3], r)) --n;
     int top = p.n_grid - 2;
@@ -554,6 +556,15 @@ struct Exit {
     int next;
     int axis;
 };
+
+// put the crossing coordinate of x exactly onto its plane (selects: an
+// indexed store would place x in local memory)
+__device__ __forceinline__ void snap(const Exit& e, double x[3])
+{
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+        if (e.axis == a) x[a] = e.plane;
+}
 
 // layer containing z for entries through a side face: largest j with
 // zb[j] <= z, clamped to [0, L-1]
@@ -931,8 +942,16 @@ __device__ __forceinline__ LayerBox layer_box(const Params<R>& p, int vol)
 template <typename R>
 __device__ __forceinline__ bool inside_box(const Params<R>& p, const LayerBox& b, const double x1[3])
 {
-    const long long k0 = ord_key(x1[0]), k1 = ord_key(x1[1]), k2 = ord_key(x1[2]);
-    return k2 > b.zlo && k2 < b.zhi && k0 > p.kxy[0] && k0 < p.kxy[1] && k1 > p.kxy[2] && k1 < p.kxy[3];
+    const long long k2 = ord_key(x1[2]);
+    return k2 > b.zlo && k2 < b.zhi && inside_walls(p, x1);
+}
+
+// x1 lies more than kChordMargin inside a layer's side walls
+template <typename R>
+__device__ __forceinline__ bool inside_walls(const Params<R>& p, const double x1[3])
+{
+    const long long k0 = ord_key(x1[0]), k1 = ord_key(x1[1]);
+    return k0 > p.kxy[0] && k0 < p.kxy[1] && k1 > p.kxy[2] && k1 < p.kxy[3];
 }
 
 // n substeps of length hs (the caller derives both from h_max); the chord
@@ -963,7 +982,7 @@ __device__ __forceinline__ double propagate_field(const Params<R>& p, int charge
                 const R h2r = R(h2);
                 rk4(p, R(kq), x, u, h2r, mdiv(h2r, R(6)), x1, u1);
                 *evals += 1;
-                if (e.axis >= 0) x1[e.axis] = e.plane;
+                snap(e, x1);
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
                     x[a] = x1[a];

@@ -230,11 +230,15 @@ __device__ __forceinline__ int transport_part(const Params<R>& p, TrackReg<R>& t
         // sections and the draw state before the propagation.
         const R xsel = draw<R>(dr) * sig_tot;
         R c = R(0);
-        for (int i = 0; i < nproc; ++i) {
-            c += sig[i];
-            if (lt_pos(xsel, c)) {
-                proc = i;
-                break;
+        bool open = true;
+#pragma unroll
+        for (int i = 0; i < (X ? 4 : 3); ++i) {
+            if (open && i < nproc) {
+                c += sig[i];
+                if (lt_pos(xsel, c)) {
+                    proc = i;
+                    open = false;
+                }
             }
         }
     }
@@ -277,25 +281,48 @@ __device__ __forceinline__ int transport_part(const Params<R>& p, TrackReg<R>& t
                 s = e.t;
 #pragma unroll
                 for (int a = 0; a < 3; ++a) t.x[a] = fma(s, ud[a], t.x[a]);
-                if (e.axis >= 0) t.x[e.axis] = e.plane;
+                snap(e, t.x);
             } else {
                 s = s_physd;
 #pragma unroll
                 for (int a = 0; a < 3; ++a) t.x[a] = x1[a];
             }
         } else {
-            // thin layers: most steps cross a plane; the navigation (with
-            // its FP32 prefilter) is cheaper than a test that mostly fails
-            e = nav_exit<G>(p, t.vol, t.x, ud);
-            if (le_pos(e.t, s_physd)) {
-                s = e.t;
-                boundary = true;
-            } else {
-                s = s_physd;
-            }
+            // Inside a layer the exit is nearly always the z plane ahead.
+            // With t the distance to that plane and s the smaller of t and
+            // the physics step, an end point x + s u more than the chord
+            // margin inside the side walls means that both walls lie beyond
+            // s (the layer is convex): the plane, or no boundary, exactly as
+            // the full navigation would decide, for one division and the
+            // three moves that the step makes anyway.
+            bool done = false;
+            if (t.vol >= 0 && nonzero(ud[2])) {
+                const bool up = gt_zero(ud[2]);
+                const double pl = p.zb[t.vol + (up ? 1 : 0)];
+                double te = mdiv(pl - t.x[2], ud[2]);
+                if (te < 0.0) te = 0.0;
+                boundary = le_pos(te, s_physd);
+                s = boundary ? te : s_physd;
+                double x1[3];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) t.x[a] = fma(s, ud[a], t.x[a]);
-            if (boundary && e.axis >= 0) t.x[e.axis] = e.plane;
+                for (int a = 0; a < 3; ++a) x1[a] = fma(s, ud[a], t.x[a]);
+                done = inside_walls(p, x1);
+                if (done) {
+                    e.next = up ? (t.vol + 1 < p.n_layers ? t.vol + 1 : kVolWorld)
+                                : (t.vol > 0 ? t.vol - 1 : kVolWorld);
+                    t.x[0] = x1[0];
+                    t.x[1] = x1[1];
+                    t.x[2] = boundary ? pl : x1[2];
+                }
+            }
+            if (!done) {
+                e = nav_exit<G>(p, t.vol, t.x, ud);
+                boundary = le_pos(e.t, s_physd);
+                s = boundary ? e.t : s_physd;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) t.x[a] = fma(s, ud[a], t.x[a]);
+                if (boundary) snap(e, t.x);
+            }
         }
     } else {
         double smax = s_physd;
