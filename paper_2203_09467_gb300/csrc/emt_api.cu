@@ -273,10 +273,12 @@ struct emt_ctx {
     int64_t it = 0;  // step-loop iterations so far
     int64_t live_g = 0, live_c = 0;
     int64_t live_q = 0;  // pipelined schedule: interactions queued for the next iteration
-    int resident_blocks = 0;
-    int resident_a = 0, resident_b = 0;  // split schedule: transport, interaction kernels
-    int persist_grid = 0;                // persistent step loop: resident blocks of the cooperative launch
-    int resident_p = 0;                  // pipelined schedule: resident blocks of the step kernel
+    // resident blocks of the step kernels without and with a field
+    int resident_blocks[2] = {0, 0};  // fused schedule
+    int resident_a[2] = {0, 0};       // split schedule: transport kernel
+    int resident_b = 0;               // split schedule: interaction kernel
+    int resident_p[2] = {0, 0};       // pipelined schedule
+    int persist_grid[2] = {0, 0};     // persistent step loop (cooperative launch)
     long long wait_cycles = 0;           // bound of one grid-barrier wait, SM clock cycles
     int block = 128;
     // host event table
@@ -755,14 +757,14 @@ emt_status run_loop(emt_ctx* c, int32_t max_iterations, emt_run_stats* st)
         // warp-sized ones (a block for every warp chunk while blocks last)
         const int per = c->plan.split && c->opt.max_active <= 0 ? 32 : c->block;
         int64_t chunks = (c->live_g + per - 1) / per + (c->live_c + per - 1) / per;
-        int grid = (int)std::max<int64_t>(1, std::min<int64_t>(chunks, c->resident_blocks));
+        int grid = (int)std::max<int64_t>(1, std::min<int64_t>(chunks, c->resident_blocks[p.has_field]));
         EMT_CUDA(c, cudaEventRecord(c->ev0, c->stream));
         cudaError_t e =
             c->plan.pipelined
-                ? Launch<R>::step_pipe(p, side, cin, cout, cclr, c->resident_p, c->resident_b, c->block, c->stream)
+                ? Launch<R>::step_pipe(p, side, cin, cout, cclr, c->resident_p[p.has_field], c->resident_b, c->block, c->stream)
             : c->plan.split
                 ? Launch<R>::step_split(p, side, cin, cout, cclr,
-                                        (int)std::max<int64_t>(1, std::min<int64_t>(chunks, c->resident_a)),
+                                        (int)std::max<int64_t>(1, std::min<int64_t>(chunks, c->resident_a[p.has_field])),
                                         c->resident_b, c->block, c->stream)
                 : Launch<R>::step(p, side, cin, cout, cclr, grid, c->block, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "step kernel launch");
@@ -812,7 +814,7 @@ emt_status run_loop(emt_ctx* c, int32_t max_iterations, emt_run_stats* st)
             }
             EMT_CUDA(c, cudaMemsetAsync(gs, 0, sizeof(GridSync), c->stream));
             EMT_CUDA(c, cudaEventRecord(c->ev0, c->stream));
-            cudaError_t e = Launch<R>::persist(p, c->it, k, gs, c->wait_cycles, c->persist_grid, c->block, c->stream);
+            cudaError_t e = Launch<R>::persist(p, c->it, k, gs, c->wait_cycles, c->persist_grid[p.has_field], c->block, c->stream);
             if (e != cudaSuccess) return cuda_fail(c, e, "persistent step loop launch");
             EMT_CUDA(c, cudaEventRecord(c->ev1, c->stream));
             GridSync h_gs;
@@ -848,11 +850,11 @@ emt_status run_loop(emt_ctx* c, int32_t max_iterations, emt_run_stats* st)
                 for (int k = 0; k < K; ++k) {
                     int side = k & 1, cin = k % 3, cout = (k + 1) % 3, cclr = (k + 2) % 3;
                     cudaError_t e = c->plan.pipelined
-                                        ? Launch<R>::step_pipe(p, side, cin, cout, cclr, c->resident_p, c->resident_b,
+                                        ? Launch<R>::step_pipe(p, side, cin, cout, cclr, c->resident_p[p.has_field], c->resident_b,
                                                                c->block, c->stream)
-                                    : c->plan.split ? Launch<R>::step_split(p, side, cin, cout, cclr, c->resident_a,
+                                    : c->plan.split ? Launch<R>::step_split(p, side, cin, cout, cclr, c->resident_a[p.has_field],
                                                                           c->resident_b, c->block, c->stream)
-                                                  : Launch<R>::step(p, side, cin, cout, cclr, c->resident_blocks,
+                                                  : Launch<R>::step(p, side, cin, cout, cclr, c->resident_blocks[p.has_field],
                                                                     c->block, c->stream);
                     if (e != cudaSuccess) {
                         cudaStreamEndCapture(c->stream, &g);
@@ -1032,30 +1034,37 @@ emt_status emt_create(const emt_options* o, emt_ctx** out)
     c->block = o->block_size ? o->block_size : 256;
     int dev_sms = 0;
     cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, o->device);
-    int per_sm = c->mixed() ? Launch<float>::max_blocks_per_sm(c->block) : Launch<double>::max_blocks_per_sm(c->block);
-    c->resident_blocks = std::max(1, dev_sms * per_sm);
-    if (c->plan.split) {
-        auto blocks = [&](int which) {
-            return c->mixed() ? Launch<float>::max_blocks_split(c->block, which)
-                              : Launch<double>::max_blocks_split(c->block, which);
-        };
-        c->resident_a = std::max(1, dev_sms * blocks(0));
-        c->resident_b = std::max(1, dev_sms * blocks(1));
+    auto resident = [&](auto per_sm_f, auto per_sm_d) {
+        return std::max(1, dev_sms * (c->mixed() ? per_sm_f() : per_sm_d()));
+    };
+    for (int f = 0; f < 2; ++f) {
+        const bool field = f != 0;
+        const int bs = c->block;
+        c->resident_blocks[f] = resident([&] { return Launch<float>::max_blocks_per_sm(bs, field); },
+                                         [&] { return Launch<double>::max_blocks_per_sm(bs, field); });
+        if (c->plan.split)
+            c->resident_a[f] = resident([&] { return Launch<float>::max_blocks_split(bs, 0, field); },
+                                        [&] { return Launch<double>::max_blocks_split(bs, 0, field); });
         if (c->plan.pipelined)
-            c->resident_p = std::max(1, dev_sms * (c->mixed() ? Launch<float>::max_blocks_pipe(c->block)
-                                                              : Launch<double>::max_blocks_pipe(c->block)));
+            c->resident_p[f] = resident([&] { return Launch<float>::max_blocks_pipe(bs, field); },
+                                        [&] { return Launch<double>::max_blocks_pipe(bs, field); });
     }
+    if (c->plan.split)
+        c->resident_b = resident([&] { return Launch<float>::max_blocks_split(c->block, 1, false); },
+                                 [&] { return Launch<double>::max_blocks_split(c->block, 1, false); });
     if (o->loop_mode == EMT_LOOP_PERSISTENT) {
         int coop = 0, clock_khz = 0;
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, o->device);
         cudaDeviceGetAttribute(&clock_khz, cudaDevAttrClockRate, o->device);
-        const int per = c->mixed() ? Launch<float>::persist_blocks_per_sm(c->block)
-                                   : Launch<double>::persist_blocks_per_sm(c->block);
-        if (!coop || per < 1 || clock_khz < 1) {
-            why = "the device cannot run the persistent step loop (cooperative launch)";
-            return bail(EMT_ERR_INVALID_ARG);
+        for (int f = 0; f < 2; ++f) {
+            const int per = c->mixed() ? Launch<float>::persist_blocks_per_sm(c->block, f != 0)
+                                       : Launch<double>::persist_blocks_per_sm(c->block, f != 0);
+            if (!coop || per < 1 || clock_khz < 1) {
+                why = "the device cannot run the persistent step loop (cooperative launch)";
+                return bail(EMT_ERR_INVALID_ARG);
+            }
+            c->persist_grid[f] = dev_sms * per;
         }
-        c->persist_grid = dev_sms * per;
         c->wait_cycles = (long long)(kPersistWaitMs * (double)clock_khz);
     }
     c->slot_id.assign(pl.max_events, 0);
@@ -1790,7 +1799,7 @@ extern "C" emt_status emt_transport_static(int32_t device, uint32_t seed, const 
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     const int block = 256;
-    const int resident = std::max(1, sms * Launch<double>::max_blocks_per_sm(block));
+    const int resident = std::max(1, sms * Launch<double>::max_blocks_per_sm(block, p.has_field != 0));
     int64_t live_g = h_cnt.n[0], live_c = h_cnt.n[1];
     unsigned long long steps[2] = {0, 0}, last_steps = 0;
     for (int64_t it = 0; live_g + live_c > 0; ++it) {

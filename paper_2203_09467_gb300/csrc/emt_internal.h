@@ -51,23 +51,24 @@ struct Launch {
                                   const uint64_t* uid, const int32_t* slot, cudaStream_t st);
     static cudaError_t get_tracks(const Params<R>& p, int side, int nG, int nC, double* rec, uint64_t* uid,
                                   int32_t* slot, cudaStream_t st);
-    static int max_blocks_per_sm(int block);
+    // resident blocks per SM of each kernel, with or without a field
+    static int max_blocks_per_sm(int block, bool field);
     // split schedule: transport kernel then interaction kernel
     static cudaError_t step_split(const Params<R>& p, int side, int cin, int cout, int cclr, int grid_a, int grid_b,
                                   int block, cudaStream_t st);
-    static int max_blocks_split(int block, int which);
+    static int max_blocks_split(int block, int which, bool field);
     // pipelined schedule: one kernel per step (plus the two sorting launches
     // of the charged tracks in a field, on grid_sort blocks)
     static cudaError_t step_pipe(const Params<R>& p, int side, int cin, int cout, int cclr, int grid, int grid_sort,
                                  int block, cudaStream_t st);
-    static int max_blocks_pipe(int block);
+    static int max_blocks_pipe(int block, bool field);
     // host spill: append n tracks of the spill buffer to side `side`
     static cudaError_t unspill(const Params<R>& p, int side, int cs, int n, cudaStream_t st);
     // persistent step loop (fused schedule, cooperative launch of `grid`
     // resident blocks): up to max_steps steps from global iteration it0
     static cudaError_t persist(const Params<R>& p, long long it0, int max_steps, GridSync* gs,
                                long long limit_cycles, int grid, int block, cudaStream_t st);
-    static int persist_blocks_per_sm(int block);
+    static int persist_blocks_per_sm(int block, bool field);
 };
 
 // diagnostics: a bounded grid wait that is never released (on `blocks`

@@ -2,104 +2,114 @@
 // once per precision in its own translation unit (different FMA flags).
 #pragma once
 
+#include <type_traits>
+
 #include "emt_internal.h"
 #include "emt_step.cuh"
 
 namespace emt {
 
-// the physics options (multiple scattering, angular distributions,
-// Rayleigh) select their own kernel instantiations
-template <typename R>
-static bool extended(const Params<R>& p)
+template <int V>
+using Int = std::integral_constant<int, V>;
+template <bool V>
+using Bool = std::integral_constant<bool, V>;
+
+// Calls fn(geometry, field, options) with the kernel instantiation's
+// template arguments as constants: the geometry kind, whether a field is on,
+// and whether the physics options (multiple scattering, angular
+// distributions, Rayleigh) may be on.
+template <typename Fn>
+static cudaError_t with_variant(bool cylinders, bool field, bool options, Fn fn)
 {
-    return (p.mask & (kProcMsc | kProcAngular | kProcRayleigh)) != 0u;
+    auto with_options = [&](auto g, auto f) { return options ? fn(g, f, Bool<true>{}) : fn(g, f, Bool<false>{}); };
+    auto with_field = [&](auto g) { return field ? with_options(g, Bool<true>{}) : with_options(g, Bool<false>{}); };
+    return cylinders ? with_field(Int<kGeomCylinders>{}) : with_field(Int<kGeomLayers>{});
 }
 
-template <typename R, int BS, int G>
-static void launch_fused(const Params<R>& p, int side, int cin, int cout, int cclr, int grid, cudaStream_t st)
+template <typename R, typename Fn>
+static cudaError_t with_variant(const Params<R>& p, Fn fn)
 {
-    if (extended(p))
-        k_step<R, BS, G, true><<<grid, BS, 0, st>>>(p, side, cin, cout, cclr);
-    else
-        k_step<R, BS, G, false><<<grid, BS, 0, st>>>(p, side, cin, cout, cclr);
+    return with_variant(p.geom == kGeomCylinders, p.has_field != 0,
+                        (p.mask & (kProcMsc | kProcAngular | kProcRayleigh)) != 0u, fn);
+}
+
+// calls fn(block size) for the supported sizes
+template <typename Fn>
+static cudaError_t with_block(int block, Fn fn)
+{
+    if (block == 128) return fn(Int<128>{});
+    if (block == 256) return fn(Int<256>{});
+    return cudaErrorInvalidValue;
+}
+
+// Smallest number of resident blocks per SM over the geometry kinds and
+// options, with or without a field; kernel(geometry, field, options) names
+// the instantiation.  0 on failure.
+template <typename Fn>
+static int min_blocks(int block, bool field, Fn kernel)
+{
+    int least = 1 << 30;
+    for (int k = 0; k < 4; ++k) {
+        int n = 0;
+        const cudaError_t e = with_variant((k & 1) != 0, field, (k & 2) != 0, [&](auto g, auto f, auto x) {
+            return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel(g, f, x), block, 0);
+        });
+        if (e != cudaSuccess) return 0;
+        if (n < least) least = n;
+    }
+    return least;
 }
 
 template <typename R>
 cudaError_t Launch<R>::step(const Params<R>& p, int side, int cin, int cout, int cclr, int grid, int block,
                             cudaStream_t st)
 {
-    const bool cyl = p.geom == kGeomCylinders;
-    if (block == 128) {
-        if (cyl)
-            launch_fused<R, 128, kGeomCylinders>(p, side, cin, cout, cclr, grid, st);
-        else
-            launch_fused<R, 128, kGeomLayers>(p, side, cin, cout, cclr, grid, st);
-    } else if (block == 256) {
-        if (cyl)
-            launch_fused<R, 256, kGeomCylinders>(p, side, cin, cout, cclr, grid, st);
-        else
-            launch_fused<R, 256, kGeomLayers>(p, side, cin, cout, cclr, grid, st);
-    } else {
-        return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
+    return with_block(block, [&](auto bs) {
+        return with_variant(p, [&](auto g, auto f, auto x) {
+            k_step<R, bs.value, g.value, f.value, x.value><<<grid, bs.value, 0, st>>>(p, side, cin, cout, cclr);
+            return cudaGetLastError();
+        });
+    });
 }
 
-template <typename R, int BS, int G, bool X>
-static cudaError_t launch_persist_x(const Params<R>& p, long long it0, int max_steps, GridSync* gs,
-                                   long long limit_cycles, int grid, cudaStream_t st)
+template <typename R>
+int Launch<R>::max_blocks_per_sm(int block, bool field)
 {
-    Params<R> pc = p;
-    void* args[] = {&pc, &it0, &max_steps, &gs, &limit_cycles};
-    return cudaLaunchCooperativeKernel((const void*)k_persist<R, BS, G, X>, dim3(grid), dim3(BS), args, 0, st);
+    int n = 0;
+    with_block(block, [&](auto bs) {
+        n = min_blocks(bs.value, field,
+                       [](auto g, auto f, auto x) { return k_step<R, decltype(bs)::value, g.value, f.value, x.value>; });
+        return cudaSuccess;
+    });
+    return n > 0 ? n : 1;
 }
 
 template <typename R>
 cudaError_t Launch<R>::persist(const Params<R>& p, long long it0, int max_steps, GridSync* gs,
                                long long limit_cycles, int grid, int block, cudaStream_t st)
 {
-    const bool cyl = p.geom == kGeomCylinders;
-    const bool x = extended(p);
-    if (block == 128) {
-        if (cyl)
-            return x ? launch_persist_x<R, 128, kGeomCylinders, true>(p, it0, max_steps, gs, limit_cycles, grid, st)
-                     : launch_persist_x<R, 128, kGeomCylinders, false>(p, it0, max_steps, gs, limit_cycles, grid, st);
-        return x ? launch_persist_x<R, 128, kGeomLayers, true>(p, it0, max_steps, gs, limit_cycles, grid, st)
-                 : launch_persist_x<R, 128, kGeomLayers, false>(p, it0, max_steps, gs, limit_cycles, grid, st);
-    }
-    if (block == 256) {
-        if (cyl)
-            return x ? launch_persist_x<R, 256, kGeomCylinders, true>(p, it0, max_steps, gs, limit_cycles, grid, st)
-                     : launch_persist_x<R, 256, kGeomCylinders, false>(p, it0, max_steps, gs, limit_cycles, grid, st);
-        return x ? launch_persist_x<R, 256, kGeomLayers, true>(p, it0, max_steps, gs, limit_cycles, grid, st)
-                 : launch_persist_x<R, 256, kGeomLayers, false>(p, it0, max_steps, gs, limit_cycles, grid, st);
-    }
-    return cudaErrorInvalidValue;
+    Params<R> pc = p;
+    void* args[] = {&pc, &it0, &max_steps, &gs, &limit_cycles};
+    return with_block(block, [&](auto bs) {
+        return with_variant(p, [&](auto g, auto f, auto x) {
+            return cudaLaunchCooperativeKernel((const void*)k_persist<R, bs.value, g.value, f.value, x.value>,
+                                               dim3(grid), dim3(bs.value), args, 0, st);
+        });
+    });
 }
 
-// resident blocks per SM of the persistent kernel, the smallest over its
-// instantiations (every block of a cooperative launch must be resident)
-template <typename R, int BS>
-static int min_blocks_persist()
-{
-    int n[4] = {0, 0, 0, 0};
-    cudaError_t e[4];
-    e[0] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[0], k_persist<R, BS, kGeomLayers, false>, BS, 0);
-    e[1] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[1], k_persist<R, BS, kGeomCylinders, false>, BS, 0);
-    e[2] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[2], k_persist<R, BS, kGeomLayers, true>, BS, 0);
-    e[3] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[3], k_persist<R, BS, kGeomCylinders, true>, BS, 0);
-    int m = 1 << 30;
-    for (int k = 0; k < 4; ++k) {
-        if (e[k] != cudaSuccess) return 0;
-        if (n[k] < m) m = n[k];
-    }
-    return m;
-}
-
+// every block of a cooperative launch must be resident
 template <typename R>
-int Launch<R>::persist_blocks_per_sm(int block)
+int Launch<R>::persist_blocks_per_sm(int block, bool field)
 {
-    return block == 128 ? min_blocks_persist<R, 128>() : min_blocks_persist<R, 256>();
+    int n = 0;
+    with_block(block, [&](auto bs) {
+        n = min_blocks(bs.value, field, [](auto g, auto f, auto x) {
+            return k_persist<R, decltype(bs)::value, g.value, f.value, x.value>;
+        });
+        return cudaSuccess;
+    });
+    return n;
 }
 
 template <typename R>
@@ -139,180 +149,94 @@ cudaError_t Launch<R>::get_tracks(const Params<R>& p, int side, int nG, int nC, 
     return cudaGetLastError();
 }
 
-// resident blocks per SM of the fused kernel, the smallest over its
-// instantiations (geometry kind x physics options)
-template <typename R, int BS>
-static int min_blocks_fused()
-{
-    int n[4] = {0, 0, 0, 0};
-    cudaError_t e[4];
-    e[0] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[0], k_step<R, BS, kGeomLayers, false>, BS, 0);
-    e[1] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[1], k_step<R, BS, kGeomCylinders, false>, BS, 0);
-    e[2] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[2], k_step<R, BS, kGeomLayers, true>, BS, 0);
-    e[3] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[3], k_step<R, BS, kGeomCylinders, true>, BS, 0);
-    int m = 1 << 30;
-    for (int k = 0; k < 4; ++k) {
-        if (e[k] != cudaSuccess) return 1;
-        if (n[k] < m) m = n[k];
-    }
-    return m > 0 ? m : 1;
-}
-
-template <typename R>
-int Launch<R>::max_blocks_per_sm(int block)
-{
-    return block == 128 ? min_blocks_fused<R, 128>() : min_blocks_fused<R, 256>();
-}
-
 }  // namespace emt
 
 #include "emt_split.cuh"
 
 namespace emt {
 
-template <typename R, int BS, bool S, bool X>
-static void launch_split_x(const Params<R>& p, int side, int cin, int cout, int cclr, int grid_a, int grid_b,
-                           cudaStream_t st)
+// charged tracks of a step in a field sorted by expected substep count (the
+// transport kernels take them in that order)
+template <typename R>
+static void launch_sort(const Params<R>& p, int side, int cin, int grid, cudaStream_t st)
 {
-    if (!S && p.has_field) {
-        // charged tracks sorted by expected substep count (k_transport takes
-        // them in that order)
-        k_sort_keys<R><<<grid_b, 256, 0, st>>>(p, side, cin);
-        k_sort_order<R><<<grid_b, 256, 0, st>>>(p, cin);
-    }
-    if (p.geom == kGeomCylinders)
-        k_transport<R, BS, kGeomCylinders, S, X><<<grid_a, BS, 0, st>>>(p, side, cin, cout, cclr);
-    else
-        k_transport<R, BS, kGeomLayers, S, X><<<grid_a, BS, 0, st>>>(p, side, cin, cout, cclr);
-    k_interact<R, BS, S, X><<<grid_b, BS, 0, st>>>(p, side, cin, cout);
+    k_sort_keys<R><<<grid, 256, 0, st>>>(p, side, cin);
+    k_sort_order<R><<<grid, 256, 0, st>>>(p, cin);
 }
 
-template <typename R, int BS, bool S>
-static void launch_split(const Params<R>& p, int side, int cin, int cout, int cclr, int grid_a, int grid_b,
-                         cudaStream_t st)
+template <typename R, bool S>
+static cudaError_t launch_split(const Params<R>& p, int side, int cin, int cout, int cclr, int grid_a, int grid_b,
+                                int block, cudaStream_t st)
 {
-    if (extended(p))
-        launch_split_x<R, BS, S, true>(p, side, cin, cout, cclr, grid_a, grid_b, st);
-    else
-        launch_split_x<R, BS, S, false>(p, side, cin, cout, cclr, grid_a, grid_b, st);
+    return with_block(block, [&](auto bs) {
+        return with_variant(p, [&](auto g, auto f, auto x) {
+            if (!S && f.value) launch_sort(p, side, cin, grid_b, st);
+            k_transport<R, bs.value, g.value, f.value, S, x.value>
+                <<<grid_a, bs.value, 0, st>>>(p, side, cin, cout, cclr);
+            k_interact<R, bs.value, S, x.value><<<grid_b, bs.value, 0, st>>>(p, side, cin, cout);
+            return cudaGetLastError();
+        });
+    });
 }
 
 template <typename R>
 cudaError_t Launch<R>::step_split(const Params<R>& p, int side, int cin, int cout, int cclr, int grid_a, int grid_b,
                                   int block, cudaStream_t st)
 {
-    const bool sel = p.max_active > 0;
-    if (block == 128) {
-        if (sel)
-            launch_split<R, 128, true>(p, side, cin, cout, cclr, grid_a, grid_b, st);
-        else
-            launch_split<R, 128, false>(p, side, cin, cout, cclr, grid_a, grid_b, st);
-    } else if (block == 256) {
-        if (sel)
-            launch_split<R, 256, true>(p, side, cin, cout, cclr, grid_a, grid_b, st);
-        else
-            launch_split<R, 256, false>(p, side, cin, cout, cclr, grid_a, grid_b, st);
-    } else {
-        return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
+    return p.max_active > 0 ? launch_split<R, true>(p, side, cin, cout, cclr, grid_a, grid_b, block, st)
+                            : launch_split<R, false>(p, side, cin, cout, cclr, grid_a, grid_b, block, st);
 }
 
 // resident blocks per SM of the split kernels (which 0: transport, 1:
-// interaction), the smallest over the instantiations
-template <typename R, int BS>
-static int min_blocks_split(int which)
-{
-    int n[8];
-    cudaError_t e[8];
-    int k = 0;
-    if (which == 0) {
-        e[k] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[k], k_transport<R, BS, kGeomLayers, false, false>, BS, 0), ++k;
-        e[k] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[k], k_transport<R, BS, kGeomCylinders, false, false>, BS, 0), ++k;
-        e[k] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[k], k_transport<R, BS, kGeomLayers, true, false>, BS, 0), ++k;
-        e[k] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[k], k_transport<R, BS, kGeomCylinders, true, false>, BS, 0), ++k;
-        e[k] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[k], k_transport<R, BS, kGeomLayers, false, true>, BS, 0), ++k;
-        e[k] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[k], k_transport<R, BS, kGeomCylinders, false, true>, BS, 0), ++k;
-        e[k] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[k], k_transport<R, BS, kGeomLayers, true, true>, BS, 0), ++k;
-        e[k] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[k], k_transport<R, BS, kGeomCylinders, true, true>, BS, 0), ++k;
-    } else {
-        e[k] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[k], k_interact<R, BS, false, false>, BS, 0), ++k;
-        e[k] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[k], k_interact<R, BS, true, false>, BS, 0), ++k;
-        e[k] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[k], k_interact<R, BS, false, true>, BS, 0), ++k;
-        e[k] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[k], k_interact<R, BS, true, true>, BS, 0), ++k;
-    }
-    int m = 1 << 30;
-    for (int j = 0; j < k; ++j) {
-        if (e[j] != cudaSuccess) return 1;
-        if (n[j] < m) m = n[j];
-    }
-    return m > 0 ? m : 1;
-}
-
+// interaction)
 template <typename R>
-int Launch<R>::max_blocks_split(int block, int which)
+int Launch<R>::max_blocks_split(int block, int which, bool field)
 {
-    return block == 128 ? min_blocks_split<R, 128>(which) : min_blocks_split<R, 256>(which);
-}
-
-template <typename R, int BS, bool X>
-static void launch_pipe_x(const Params<R>& p, int side, int cin, int cout, int cclr, int grid, int grid_sort,
-                          cudaStream_t st)
-{
-    if (p.has_field) {
-        k_sort_keys<R><<<grid_sort, 256, 0, st>>>(p, side, cin);
-        k_sort_order<R><<<grid_sort, 256, 0, st>>>(p, cin);
-    }
-    if (p.geom == kGeomCylinders)
-        k_pipe<R, BS, kGeomCylinders, X><<<grid, BS, 0, st>>>(p, side, cin, cout, cclr);
-    else
-        k_pipe<R, BS, kGeomLayers, X><<<grid, BS, 0, st>>>(p, side, cin, cout, cclr);
+    int n = 0;
+    with_block(block, [&](auto bs) {
+        constexpr int kBs = decltype(bs)::value;
+        if (which == 0) {
+            const int all = min_blocks(kBs, field, [](auto g, auto f, auto x) {
+                return k_transport<R, kBs, g.value, f.value, false, x.value>;
+            });
+            const int selected = min_blocks(kBs, field, [](auto g, auto f, auto x) {
+                return k_transport<R, kBs, g.value, f.value, true, x.value>;
+            });
+            n = all < selected ? all : selected;
+        } else {
+            const int all = min_blocks(kBs, field, [](auto, auto, auto x) { return k_interact<R, kBs, false, x.value>; });
+            const int selected =
+                min_blocks(kBs, field, [](auto, auto, auto x) { return k_interact<R, kBs, true, x.value>; });
+            n = all < selected ? all : selected;
+        }
+        return cudaSuccess;
+    });
+    return n > 0 ? n : 1;
 }
 
 template <typename R>
 cudaError_t Launch<R>::step_pipe(const Params<R>& p, int side, int cin, int cout, int cclr, int grid, int grid_sort,
                                  int block, cudaStream_t st)
 {
-    const bool x = extended(p);
-    if (block == 128) {
-        if (x)
-            launch_pipe_x<R, 128, true>(p, side, cin, cout, cclr, grid, grid_sort, st);
-        else
-            launch_pipe_x<R, 128, false>(p, side, cin, cout, cclr, grid, grid_sort, st);
-    } else if (block == 256) {
-        if (x)
-            launch_pipe_x<R, 256, true>(p, side, cin, cout, cclr, grid, grid_sort, st);
-        else
-            launch_pipe_x<R, 256, false>(p, side, cin, cout, cclr, grid, grid_sort, st);
-    } else {
-        return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-}
-
-// resident blocks per SM of the pipelined kernel, the smallest over its
-// instantiations
-template <typename R, int BS>
-static int min_blocks_pipe()
-{
-    int n[4] = {0, 0, 0, 0};
-    cudaError_t e[4];
-    e[0] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[0], k_pipe<R, BS, kGeomLayers, false>, BS, 0);
-    e[1] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[1], k_pipe<R, BS, kGeomCylinders, false>, BS, 0);
-    e[2] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[2], k_pipe<R, BS, kGeomLayers, true>, BS, 0);
-    e[3] = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n[3], k_pipe<R, BS, kGeomCylinders, true>, BS, 0);
-    int m = 1 << 30;
-    for (int k = 0; k < 4; ++k) {
-        if (e[k] != cudaSuccess) return 1;
-        if (n[k] < m) m = n[k];
-    }
-    return m > 0 ? m : 1;
+    return with_block(block, [&](auto bs) {
+        return with_variant(p, [&](auto g, auto f, auto x) {
+            if (f.value) launch_sort(p, side, cin, grid_sort, st);
+            k_pipe<R, bs.value, g.value, f.value, x.value><<<grid, bs.value, 0, st>>>(p, side, cin, cout, cclr);
+            return cudaGetLastError();
+        });
+    });
 }
 
 template <typename R>
-int Launch<R>::max_blocks_pipe(int block)
+int Launch<R>::max_blocks_pipe(int block, bool field)
 {
-    return block == 128 ? min_blocks_pipe<R, 128>() : min_blocks_pipe<R, 256>();
+    int n = 0;
+    with_block(block, [&](auto bs) {
+        n = min_blocks(bs.value, field,
+                       [](auto g, auto f, auto x) { return k_pipe<R, decltype(bs)::value, g.value, f.value, x.value>; });
+        return cudaSuccess;
+    });
+    return n > 0 ? n : 1;
 }
 
 }  // namespace emt
@@ -328,15 +252,15 @@ int Launch<R>::max_blocks_pipe(int block)
                                                const int32_t*, cudaStream_t);                                     \
     template cudaError_t Launch<R>::get_tracks(const Params<R>&, int, int, int, double*, uint64_t*, int32_t*,     \
                                                cudaStream_t);                                                     \
-    template int Launch<R>::max_blocks_per_sm(int);                                                               \
+    template int Launch<R>::max_blocks_per_sm(int, bool);                                                               \
     template cudaError_t Launch<R>::unspill(const Params<R>&, int, int, int, cudaStream_t);
 #define EMT_INSTANTIATE_PERSIST(R)                                                                                  \
     template cudaError_t Launch<R>::persist(const Params<R>&, long long, int, GridSync*, long long, int, int,     \
                                             cudaStream_t);                                                        \
-    template int Launch<R>::persist_blocks_per_sm(int);
+    template int Launch<R>::persist_blocks_per_sm(int, bool);
 #define EMT_INSTANTIATE_SPLIT(R)                                                                                    \
     template cudaError_t Launch<R>::step_split(const Params<R>&, int, int, int, int, int, int, int, cudaStream_t); \
-    template int Launch<R>::max_blocks_split(int, int);
+    template int Launch<R>::max_blocks_split(int, int, bool);
 #define EMT_INSTANTIATE_PIPE(R)                                                                                     \
     template cudaError_t Launch<R>::step_pipe(const Params<R>&, int, int, int, int, int, int, int, cudaStream_t);  \
-    template int Launch<R>::max_blocks_pipe(int);
+    template int Launch<R>::max_blocks_pipe(int, bool);

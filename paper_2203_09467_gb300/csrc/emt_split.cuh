@@ -28,16 +28,18 @@ __device__ __forceinline__ uint32_t pack_tvm(int type, int vol, int model)
 // policy; both kernels count their outputs' energy classes for the next
 // step's selection.
 // Resident threads per SM the transport kernel is compiled for (its
-// register budget), measured on GB300.  FP64: 512 (128 registers, almost no
-// spills).  In a field the RK4 substeps keep many doubles live; at 768
-// threads (80 registers) their spills share the FP64 unit's issue queue,
-// and the field transport runs 13% slower.  Without a field 768 was 1% faster,
-// but there the pipelined schedule is used.  Mixed precision: 640 (768
-// measured 14% slower in the field, 2% faster on the cylinder problem).
-template <typename R>
+// register budget), measured on GB300.
+// Field: FP64 512 (128 registers), mixed 640.  The RK4 substeps keep many
+// doubles live: at 768 threads (80 registers) their spills share the FP64
+// unit's issue queue and the field transport ran 13-14% slower.
+// No field: 768 (80 registers, a few spills).  The step is bound by the
+// latency of its dependent chain, so more warps pay: 10,000-event
+// calorimeter at 768 against 512 threads, mixed 22.12 against 22.99 ms; the
+// cylinder shells lose 0.5% in FP64 (23.38 against 23.26 ms).
+template <typename R, bool F>
 constexpr int transport_threads_per_sm()
 {
-    return sizeof(R) == 8 ? 512 : 640;
+    return F ? (sizeof(R) == 8 ? 512 : 640) : 768;
 }
 
 // Phase A of one track in the transport kernel (every lane of the warp
@@ -46,7 +48,7 @@ constexpr int transport_threads_per_sm()
 // interacting track (into iq, counted in *n_iq) for the interaction phase.
 // count_queued: a queued track's step is counted now (split schedule) or
 // when its interaction is committed (pipelined schedule).
-template <int G, bool X, typename R>
+template <int G, bool F, bool X, typename R>
 __device__ __forceinline__ void transport_lane(const Params<R>& p, const Tracks<R>& qo, Counters* co,
                                                const InterQueue<R>& iq, int* n_iq, bool count_queued, int lane,
                                                TrackReg<R>& t, bool active, bool held, long long src, unsigned* eh,
@@ -63,8 +65,8 @@ __device__ __forceinline__ void transport_lane(const Params<R>& p, const Tracks<
         copy_out(t, o);
     } else if (active) {
         bool alive;
-        model = transport_part<G, X>(p, t, fx, alive);
-        tally.substeps += (unsigned)fx.substeps;
+        model = transport_part<G, F, X>(p, t, fx, alive);
+        if constexpr (F) tally.substeps += (unsigned)fx.substeps;
         finish = model == kNoInteraction;
         if (finish) finish_step(p, t, alive, fx, o);
     }
@@ -189,8 +191,8 @@ __global__ void __launch_bounds__(256) k_sort_order(Params<R> p, int cin)
     }
 }
 
-template <typename R, int BS, int G, bool S, bool X>
-__global__ void __launch_bounds__(BS, transport_threads_per_sm<R>() / BS)
+template <typename R, int BS, int G, bool F, bool S, bool X>
+__global__ void __launch_bounds__(BS, transport_threads_per_sm<R, F>() / BS)
     k_transport(Params<R> p, int side, int cin, int cout, int cclr)
 {
     __shared__ int s_chunk;
@@ -210,7 +212,7 @@ __global__ void __launch_bounds__(BS, transport_threads_per_sm<R>() / BS)
     // In a field the charged tracks (tens of RK4 substeps per step) are
     // handed out before the photons, so that the cheap photon work fills
     // the end of the launch instead of the expensive charged work.
-    const bool charged_first = p.has_field != 0;
+    constexpr bool charged_first = F;
 
     if constexpr (!select) {
         // Chunks of one warp, taken by each warp on its own (no block
@@ -219,7 +221,6 @@ __global__ void __launch_bounds__(BS, transport_threads_per_sm<R>() / BS)
         // k_sort_order (most expensive first).
         const int chunksG = (nG + 31) >> 5;
         const int chunksC = (nC + 31) >> 5;
-        const bool sorted = p.has_field != 0;
         StepTally tally;
         // The first chunk of a warp is fixed: warp 0 of every block before
         // warp 1 of any, so that the first (in a field: the most expensive)
@@ -235,15 +236,15 @@ __global__ void __launch_bounds__(BS, transport_threads_per_sm<R>() / BS)
                                            : (charged_first ? chunk : chunk - chunksG);
             long long i = (long long)local * 32 + lane;
             const bool active = i < (photon_chunk ? nG : nC);
-            if (sorted && !photon_chunk && active) i = p.sperm[i];
+            if (charged_first && !photon_chunk && active) i = p.sperm[i];
             const long long src = photon_chunk ? i : Q - nC + i;
             TrackReg<R> t;
             if (active) load_track(qi, src, t);
-            transport_lane<G, X>(p, qo, co, p.iq, &p.cnt[cin].n_int, true, lane, t, active, false, src, nullptr,
+            transport_lane<G, F, X>(p, qo, co, p.iq, &p.cnt[cin].n_int, true, lane, t, active, false, src, nullptr,
                                  tally);
             chunk = __shfl_sync(0xFFFFFFFFu, next, 0);
         }
-        flush_tally(p, lane, tally);
+        flush_tally<F>(p, lane, tally);
         return;
     }
 
@@ -335,9 +336,9 @@ __global__ void __launch_bounds__(BS, transport_threads_per_sm<R>() / BS)
             const unsigned mh = __ballot_sync(0xFFFFFFFFu, held);
             if (lane == 0 && mh) atomicAdd(&p.total_steps[2], (unsigned long long)__popc(mh));
         }
-        transport_lane<G, X>(p, qo, co, p.iq, &p.cnt[cin].n_int, true, lane, t, active, held, src, s_eh, tally);
+        transport_lane<G, F, X>(p, qo, co, p.iq, &p.cnt[cin].n_int, true, lane, t, active, held, src, s_eh, tally);
     }
-    flush_tally(p, lane, tally);
+    flush_tally<F>(p, lane, tally);
     if constexpr (select) {
         __syncthreads();
         for (int b = threadIdx.x; b < kEBins; b += BS)
@@ -540,23 +541,22 @@ __global__ void __launch_bounds__(BS, 512 / BS) k_interact(Params<R> p, int side
     interact_chunks<R, BS, X, false>(p, p.q[side], p.q[side ^ 1], &p.cnt[cout], cin, p.iq, p.cnt[cin].n_int,
                                      p.Q - ntot, 2 * ntot <= p.Q, p.iq, nullptr, select ? s_eh : nullptr, s_chunk,
                                      count, offset, perm, tally);
-    flush_tally(p, threadIdx.x & 31, tally);
+    flush_tally<false>(p, threadIdx.x & 31, tally);
     if constexpr (select) {
         for (int b = threadIdx.x; b < kEBins; b += BS)
             if (s_eh[b]) atomicAdd(&p.ehist[(size_t)cout * kEBins + b], s_eh[b]);
     }
 }
 
-// Resident threads per SM of the pipelined kernel (its register budget).
-// FP64: 512 (128 registers, the interaction phase without spills); mixed
-// precision: 768 (about 80 registers, little spilled), whose extra
-// resident warps hide more of the transport phase's latency (+3% on the
-// calorimeter against 512; the FP64 kernel at 768 spills ~500 bytes a
-// thread and gains nothing).
-template <typename R>
+// Resident threads per SM of the pipelined kernel (its register budget), as
+// for the transport kernel: FP64 in a field 512 (at 768 it spills about 500
+// bytes a thread and gains nothing), otherwise 768 (80 registers).  FP64
+// calorimeter of 10,000 events at 768 against 512 threads: 46.3 against
+// 48.0 ms.
+template <typename R, bool F>
 constexpr int pipe_threads_per_sm()
 {
-    return sizeof(R) == 8 ? 512 : 768;
+    return F && sizeof(R) == 8 ? 512 : 768;
 }
 
 // Pipelined schedule: one kernel per step-loop iteration.  Its blocks
@@ -569,8 +569,8 @@ constexpr int pipe_threads_per_sm()
 // one after the other; an interacting track's step simply completes one
 // iteration later.  Each input track and each queued record owns one output
 // slot; a record with two outputs takes a growth token from the rest.
-template <typename R, int BS, int G, bool X>
-__global__ void __launch_bounds__(BS, pipe_threads_per_sm<R>() / BS)
+template <typename R, int BS, int G, bool F, bool X>
+__global__ void __launch_bounds__(BS, pipe_threads_per_sm<R, F>() / BS)
     k_pipe(Params<R> p, int side, int cin, int cout, int cclr)
 {
     constexpr int CH = BS * kInteractRecords;
@@ -601,7 +601,7 @@ __global__ void __launch_bounds__(BS, pipe_threads_per_sm<R>() / BS)
     const int lane = threadIdx.x & 31;
     const int chunksG = (nG + 31) >> 5;
     const int chunksC = (nC + 31) >> 5;
-    const bool charged_first = p.has_field != 0;
+    constexpr bool charged_first = F;
     // The first chunk of a warp is fixed, as in k_transport, starting with
     // the blocks that had no interactions to sample.
     const int grid = (int)gridDim.x;
@@ -621,10 +621,10 @@ __global__ void __launch_bounds__(BS, pipe_threads_per_sm<R>() / BS)
         const long long src = photon_chunk ? i : Q - nC + i;
         TrackReg<R> t;
         if (active) load_track(qi, src, t);
-        transport_lane<G, X>(p, qo, co, q_next, n_next, false, lane, t, active, false, src, nullptr, tally);
+        transport_lane<G, F, X>(p, qo, co, q_next, n_next, false, lane, t, active, false, src, nullptr, tally);
         chunk = __shfl_sync(0xFFFFFFFFu, next, 0);
     }
-    flush_tally(p, lane, tally);
+    flush_tally<F>(p, lane, tally);
 }
 
 }  // namespace emt

@@ -147,10 +147,10 @@ struct StepTally {
 };
 
 // every lane of the warp calls it
-template <typename R>
+template <bool F, typename R>
 __device__ __forceinline__ void flush_tally(const Params<R>& p, int lane, const StepTally& c)
 {
-    const unsigned sub = p.has_field ? __reduce_add_sync(0xFFFFFFFFu, c.substeps) : 0u;
+    const unsigned sub = F ? __reduce_add_sync(0xFFFFFFFFu, c.substeps) : 0u;
     if (lane != 0) return;
     if (c.steps) atomicAdd(&p.total_steps[0], (unsigned long long)(long long)c.steps);
     if (c.deferred) atomicAdd(&p.total_steps[1], (unsigned long long)c.deferred);
@@ -169,10 +169,11 @@ __device__ __forceinline__ void flush_tally(const Params<R>& p, int lane, const 
 //    a null interaction.
 // Returns the model to sample in phase B, or kNoInteraction.  `alive`
 // reports whether the track survives phase A.
-// G: geometry kind; X: the physics options (multiple scattering, angular
-// distributions, Rayleigh) may be on (kernels without them carry no code
-// for them)
-template <int G, bool X, typename R>
+// G: geometry kind; F: a magnetic field is on; X: the physics options
+// (multiple scattering, angular distributions, Rayleigh) may be on.  Kernels
+// without a field or without the options carry no code for them: fewer
+// registers, fewer instructions to fetch.
+template <int G, bool F, bool X, typename R>
 __device__ __forceinline__ int transport_part(const Params<R>& p, TrackReg<R>& t, Effects& fx, bool& alive)
 {
     fx.dep = 0.0;
@@ -262,7 +263,7 @@ __device__ __forceinline__ int transport_part(const Params<R>& p, TrackReg<R>& t
     bool boundary = false;
     Exit e;
     const double s_physd = to_d(s_phys);
-    if (!(charged && p.has_field)) {
+    if (!(F && charged)) {
         const double ud[3] = {to_d(t.u[0]), to_d(t.u[1]), to_d(t.u[2])};
         if constexpr (G == kGeomCylinders) {
             // cylinders (thick shells, navigation with square roots): a
@@ -324,7 +325,7 @@ __device__ __forceinline__ int transport_part(const Params<R>& p, TrackReg<R>& t
                 if (boundary) snap(e, t.x);
             }
         }
-    } else {
+    } else if constexpr (F) {
         double smax = s_physd;
         if (smax > p.max_field_step) {
             smax = p.max_field_step;
@@ -733,7 +734,7 @@ struct Staging {
 // is copied unchanged (its step counter, hence its random stream, is kept).
 // Only interactions make two outputs.  When 2n <= Q every step fits and no
 // token is counted.
-template <typename R, int BS, int G, bool X>
+template <typename R, int BS, int G, bool F, bool X>
 __device__ __forceinline__ void step_body(const Params<R>& p, int side, int cin, int cout, int cclr, int& s_chunk,
                                           Staging<R, BS>& sg)
 {
@@ -780,8 +781,8 @@ __device__ __forceinline__ void step_body(const Params<R>& p, int side, int cin,
         if (active) {
             load_track(qi, src, t);
             bool alive;
-            model = transport_part<G, X>(p, t, fx, alive);
-            tally.substeps += (unsigned)fx.substeps;
+            model = transport_part<G, F, X>(p, t, fx, alive);
+            if constexpr (F) tally.substeps += (unsigned)fx.substeps;
             if (model == kNoInteraction) {
                 finish_step(p, t, alive, fx, o);
                 live = apply_effects(p, t.ev, t.type, t.step, fx);
@@ -883,15 +884,15 @@ __device__ __forceinline__ void step_body(const Params<R>& p, int side, int cin,
         __syncthreads();
         chunk = s_chunk;
     }
-    flush_tally(p, lane, tally);
+    flush_tally<F>(p, lane, tally);
 }
 
-template <typename R, int BS, int G, bool X>
+template <typename R, int BS, int G, bool F, bool X>
 __global__ void __launch_bounds__(BS, 512 / BS) k_step(Params<R> p, int side, int cin, int cout, int cclr)
 {
     __shared__ int s_chunk;
     __shared__ Staging<R, BS> sg;
-    step_body<R, BS, G, X>(p, side, cin, cout, cclr, s_chunk, sg);
+    step_body<R, BS, G, F, X>(p, side, cin, cout, cclr, s_chunk, sg);
 }
 
 // Grid-wide barrier of a persistent kernel whose blocks are all resident
@@ -940,7 +941,7 @@ __device__ __forceinline__ bool grid_barrier(GridSync* gs, unsigned blocks, long
 // synchronization points per step, Sec. 3.2) where a step is short: the
 // tail of a run, one event at a time, a served stream at a low rate.
 // gs->iters receives the number of steps run.
-template <typename R, int BS, int G, bool X>
+template <typename R, int BS, int G, bool F, bool X>
 __global__ void __launch_bounds__(BS, 512 / BS)
     k_persist(Params<R> p, long long it0, int max_steps, GridSync* gs, long long limit_cycles)
 {
@@ -951,7 +952,7 @@ __global__ void __launch_bounds__(BS, 512 / BS)
     while (done < max_steps) {
         const long long it = it0 + done;
         const int side = (int)(it & 1), cin = (int)(it % 3), cout = (int)((it + 1) % 3), cclr = (int)((it + 2) % 3);
-        step_body<R, BS, G, X>(p, side, cin, cout, cclr, s_chunk, sg);
+        step_body<R, BS, G, F, X>(p, side, cin, cout, cclr, s_chunk, sg);
         ++done;
         if (!grid_barrier(gs, gridDim.x, limit_cycles, p.status)) return;
         if (threadIdx.x == 0) s_go = p.cnt[cout].n[0] + p.cnt[cout].n[1] > 0;
