@@ -63,32 +63,37 @@ EMT_LHD int clz64(uint64_t v)
 
 // floor((a b) / 2^64) for signed a, b
 EMT_LHD int64_t mulhi(int64_t a, int64_t b) { return (int64_t)(((i128)a * b) >> 64); }
+EMT_LHD int32_t mulhi32(int32_t a, int32_t b) { return (int32_t)(((int64_t)a * b) >> 32); }
 
-// Q0.64 coefficients 1/(n + 3), n = 0..6, rounded to nearest
+// Q0.64 coefficients 1/(n + 3) of r^n, n = 0..3, rounded to nearest,
 constexpr int64_t kC3 = 6148914691236517205ll;
 constexpr int64_t kC4 = 4611686018427387904ll;
 constexpr int64_t kC5 = 3689348814741910323ll;
 constexpr int64_t kC6 = 3074457345618258602ll;
-constexpr int64_t kC7 = 2635249153387078802ll;
-constexpr int64_t kC8 = 2305843009213693952ll;
-constexpr int64_t kC9 = 2049638230412172402ll;
+// and Q0.32 coefficients of the last three
+constexpr int32_t kC7 = 613566757;
+constexpr int32_t kC8 = 536870912;
+constexpr int32_t kC9 = 477218588;
 
 // nearest double to v 2^-F for 0 < v < 2^127 (F = 116 or 128)
 EMT_LHD double fixed_to_double(u128 v, int F)
 {
-    const uint64_t hi = (uint64_t)(v >> 64), lo = (uint64_t)v;
-    const int msb = hi ? 127 - clz64(hi) : 63 - clz64(lo);
-    const int e = msb - F;  // unbiased exponent of the result
-    uint64_t q;
-    if (msb <= 52) {
-        q = (uint64_t)v << (52 - msb);  // exact
-    } else {
-        const int sh = msb - 52;
-        q = (uint64_t)(v >> sh);
-        const u128 rest = v & (((u128)1 << sh) - 1), half = (u128)1 << (sh - 1);
-        if (rest > half || (rest == half && (q & 1))) q += 1;  // nearest, ties to even
+    // leading bit to bit 127, then round the top 53 bits
+    uint64_t hi = (uint64_t)(v >> 64), lo = (uint64_t)v;
+    int e = 127 - F;  // unbiased exponent of the result
+    if (hi == 0) {
+        hi = lo;
+        lo = 0;
+        e -= 64;
     }
-    uint64_t b = ((uint64_t)(e + 1022) << 52) + q;  // q = 2^53 carries into the exponent
+    const int s = clz64(hi);
+    e -= s;
+    hi = (hi << s) | ((lo >> 1) >> (63 - s));
+    lo <<= s;
+    uint64_t q = hi >> 11;
+    const uint32_t rest = (uint32_t)hi & 0x7FFu;
+    if (rest > 0x400u || (rest == 0x400u && (lo != 0 || (q & 1)))) q += 1;  // nearest, ties to even
+    const uint64_t b = ((uint64_t)(e + 1022) << 52) + q;  // q = 2^53 carries into the exponent
     double d;
     memcpy(&d, &b, 8);
     return d;
@@ -117,10 +122,11 @@ EMT_LHD_CALL double log_rn(double x)
     // bits of the product are the whole difference
     const int64_t R = (int64_t)((M * I) << (1 - sh));
     const int64_t r64 = R >> 4;  // r in Q0.64
-    int64_t p = kC9;
-    p = kC8 - mulhi(r64, p);
-    p = kC7 - mulhi(r64, p);
-    p = kC6 - mulhi(r64, p);
+    // P3 is needed to 2^-62 of 1; |r| <= 2^-8, so the terms from r^4 on are
+    // needed to 2^-32 and the r^3 term to 2^-40: 32-bit products
+    const int32_t r32 = (int32_t)(r64 >> 32), r39 = (int32_t)(r64 >> 25);
+    const int32_t q = kC7 - mulhi32(r32, kC8 - mulhi32(r32, kC9));
+    int64_t p = kC6 - (((int64_t)r39 * q) >> 7);
     p = kC5 - mulhi(r64, p);
     p = kC4 - mulhi(r64, p);
     p = kC3 - mulhi(r64, p);
