@@ -45,7 +45,7 @@ struct Plan {
     size_t hist, ledger, counts, live, event_id, done_ring;
     size_t grid, gridf, igrid, igridf, irs, irsf, tab, tabf, dedx, mats, bk, vacuum, x0, ray_a, scratch;
     size_t dgrid, dgridf, dtab, dtabf;
-    size_t zb, lmat, lbin;
+    size_t zb, kz, lmat, lbin;
     size_t st_ev, st_type, st_T, st_pos, st_dir, st_uid, st_slot, st_ids, st_start, st_runs;
     size_t slots_tmp, out_hist, out_summary;
     size_t iq[13];      // split schedule: interaction queue fields
@@ -109,6 +109,7 @@ Plan make_plan(const emt_options& o)
     p.ray_a = p.add(kMaxMat * sizeof(double));
     p.scratch = p.add((32 + (size_t)kMaxMat * 2 * kMaxGrid) * sizeof(double));
     p.zb = p.add((kMaxLayers + 1) * sizeof(double));
+    p.kz = p.add((kMaxLayers + 1) * 2 * sizeof(long long));
     p.lmat = p.add(kMaxLayers * sizeof(int));
     p.lbin = p.add(kMaxLayers * sizeof(int));
     const size_t P = (size_t)p.max_prim;
@@ -178,10 +179,10 @@ bool valid_options(const emt_options& o, std::string& why)
 }
 
 // Validate a geometry description and lay out its arrays: zb[n + 1] (plane
-// positions or shell radii), lm[n] (materials), lb[n] (score bins).
-// Returns an error message, or nullptr.
+// positions or shell radii), lm[n] (materials), lb[n] (score bins), and the
+// chord test's keys kz[n + 1][2] of the planes.  Returns an error message, or nullptr.
 const char* check_geometry(const emt_layer* layers, int n, const emt_world* w, int n_mat, int max_bins, double* zb,
-                           int* lm, int* lb)
+                           int* lm, int* lb, long long* kz)
 {
     if (n < 1 || n > kMaxLayers) return "layer count out of [1, 4096]";
     if (w->n_bins < 1 || w->n_bins > max_bins) return "n_bins out of [1, max_bins]";
@@ -196,6 +197,10 @@ const char* check_geometry(const emt_layer* layers, int n, const emt_world* w, i
         zb[i + 1] = zb[i] + layers[i].thickness_cm;
         lm[i] = layers[i].material;
         lb[i] = layers[i].score_bin;
+    }
+    for (int i = 0; i <= n; ++i) {
+        kz[2 * i + 0] = ord_key(zb[i] + kChordMargin);
+        kz[2 * i + 1] = ord_key(zb[i] - kChordMargin);
     }
     if (w->geometry == EMT_GEOM_LAYERS) {
         if (!(w->half_x_cm > 0.0) || !(w->half_y_cm > 0.0)) return "stack half widths";
@@ -228,7 +233,7 @@ void set_bin_guess(Params<R>& p, R lo, R hi, int bpd)
 
 // geometry, field and scoring fields of the kernel parameters
 template <typename R>
-void set_geometry(Params<R>& p, int n, const emt_world* w)
+void set_geometry(Params<R>& p, int n, const emt_world* w, const double* zb)
 {
     p.geom = w->geometry;
     p.half_z = w->half_z_cm;
@@ -239,15 +244,25 @@ void set_geometry(Params<R>& p, int n, const emt_world* w)
     p.kxy[1] = ord_key(p.hx - kChordMargin);
     p.kxy[2] = ord_key(-p.hy + kChordMargin);
     p.kxy[3] = ord_key(p.hy - kChordMargin);
+    const double stack[3][2] = {{-p.hx, p.hx}, {-p.hy, p.hy}, {zb[0], zb[n]}};
     for (int a = 0; a < 3; ++a) {
         p.wlo[a] = w->lo_cm[a];
         p.whi[a] = w->hi_cm[a];
         p.B[a] = w->B_tesla[a];
+        p.kworld[a][0] = ord_key(p.wlo[a] + kChordMargin);
+        p.kworld[a][1] = ord_key(p.whi[a] - kChordMargin);
+        p.kstack[a][0] = ord_key(stack[a][0] - kChordMargin);
+        p.kstack[a][1] = ord_key(stack[a][1] + kChordMargin);
     }
     p.bmag = std::sqrt(w->B_tesla[0] * w->B_tesla[0] + w->B_tesla[1] * w->B_tesla[1] + w->B_tesla[2] * w->B_tesla[2]);
     p.rk_delta = w->rk_delta_cm;
     p.max_field_step = w->max_field_step_cm;
     p.has_field = p.bmag > 0.0 ? 1 : 0;
+    p.baxis = -1;
+    for (int a = 0; a < 3; ++a) {
+        p.bhat[a] = p.has_field ? p.B[a] / p.bmag : 0.0;
+        if (p.has_field && p.B[(a + 1) % 3] == 0.0 && p.B[(a + 2) % 3] == 0.0) p.baxis = a;
+    }
     p.max_steps = w->max_steps;
     p.n_bins = w->n_bins;
     p.score_z = w->score_z;
@@ -418,6 +433,7 @@ void fill_common(emt_ctx* c, Params<R>& p)
     p.x0 = c->at<double>(pl.x0);
     p.ray_a = c->at<double>(pl.ray_a);
     p.zb = c->at<double>(pl.zb);
+    p.kz = c->at<long long>(pl.kz);
     p.lmat = c->at<int>(pl.lmat);
     p.lbin = c->at<int>(pl.lbin);
     p.step_bins = pl.step_bins;
@@ -1199,16 +1215,19 @@ emt_status emt_load_geometry(emt_ctx* c, const emt_layer* layers, int32_t n, con
     if (n < 1 || n > kMaxLayers) return fail(c, EMT_ERR_INVALID_ARG, "layer count out of [1, 4096]");
     std::vector<double> zb(n + 1);
     std::vector<int> lm(n), lb(n);
-    if (const char* why = check_geometry(layers, n, w, c->n_mat, c->opt.max_bins, zb.data(), lm.data(), lb.data()))
+    std::vector<long long> kz(2 * (size_t)n + 2);
+    if (const char* why =
+            check_geometry(layers, n, w, c->n_mat, c->opt.max_bins, zb.data(), lm.data(), lb.data(), kz.data()))
         return fail(c, EMT_ERR_INVALID_ARG, why);
     if (cudaSetDevice(c->opt.device) != cudaSuccess) return fail(c, EMT_ERR_CUDA, "cudaSetDevice");
     const Plan& pl = c->plan;
     EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.zb, zb.data(), sizeof(double) * (n + 1), cudaMemcpyHostToDevice, c->stream));
     EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.lmat, lm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, c->stream));
     EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.lbin, lb.data(), sizeof(int) * n, cudaMemcpyHostToDevice, c->stream));
+    EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.kz, kz.data(), sizeof(long long) * kz.size(), cudaMemcpyHostToDevice, c->stream));
     EMT_CUDA(c, cudaStreamSynchronize(c->stream));
-    set_geometry(c->pd, n, w);
-    set_geometry(c->pf, n, w);
+    set_geometry(c->pd, n, w, zb.data());
+    set_geometry(c->pf, n, w, zb.data());
     c->n_layers = n;
     c->n_bins = w->n_bins;
     drop_graph(c);
@@ -1745,12 +1764,15 @@ extern "C" emt_status emt_transport_static(int32_t device, uint32_t seed, const 
     // ---- geometry
     double zb[kMaxLayers + 1];
     int lm[kMaxLayers], lb[kMaxLayers];
-    if (check_geometry(layers, n_layers, w, n_mat, EMT_STATIC_MAX_BINS, zb, lm, lb)) return EMT_ERR_INVALID_ARG;
+    long long kz[2 * (kMaxLayers + 1)];
+    if (check_geometry(layers, n_layers, w, n_mat, EMT_STATIC_MAX_BINS, zb, lm, lb, kz)) return EMT_ERR_INVALID_ARG;
     if (cudaMemcpyAsync(pool + pl.zb, zb, sizeof(double) * (n_layers + 1), cudaMemcpyHostToDevice, st) != cudaSuccess ||
+        cudaMemcpyAsync(pool + pl.kz, kz, sizeof(long long) * 2 * (n_layers + 1), cudaMemcpyHostToDevice, st) !=
+            cudaSuccess ||
         cudaMemcpyAsync(pool + pl.lmat, lm, sizeof(int) * n_layers, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(pool + pl.lbin, lb, sizeof(int) * n_layers, cudaMemcpyHostToDevice, st) != cudaSuccess)
         return EMT_ERR_CUDA;
-    set_geometry(p, n_layers, w);
+    set_geometry(p, n_layers, w, zb);
 
     // ---- events: slots 0..n_events-1 in order; primaries read in place
     uint32_t slots[EMT_STATIC_MAX_EVENTS];

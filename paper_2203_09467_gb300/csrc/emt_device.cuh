@@ -238,13 +238,18 @@ struct Params {
     const int* lbin;
     int n_layers;
     double hx, hy;
-    // ord_key of the lateral bounds of a layer's chord test, formed once
-    // when the geometry is loaded: -hx + m, hx - m, -hy + m, hy - m
-    // (m = kChordMargin)
+    // ord_key of the bounds of the chord tests, formed once when the geometry
+    // is loaded (m = kChordMargin): a layer's side walls -hx + m, hx - m,
+    // -hy + m, hy - m and planes zb[i] + m, zb[i] - m ([n_layers + 1][2]); the
+    // world box shrunk by m and the layer stack grown by it, [axis][low, high]
     long long kxy[4];
+    const long long* kz;
+    long long kworld[3][2], kstack[3][2];
     double wlo[3], whi[3];
     double B[3];
     double bmag;
+    double bhat[3];  // B / |B|
+    int baxis;       // the axis a field along one coordinate axis has, else -1
     double rk_delta, max_field_step;
     int has_field;
     int max_steps;
@@ -814,51 +819,176 @@ __device__ __forceinline__ Exit nav_exit(const Params<R>& p, int vol, const doub
 }
 
 // ------------------------------------------------------------------ field
-// classical RK4 in path length on (x, u), du/ds = kq u x B, |p| fixed
-// during the step; u renormalised after each substep.  The direction and
-// its derivatives are evaluated in R (FP64 path: double, in the operation
-// order of the definition; mixed path: float), positions accumulate in FP64.
-template <typename R>
-__device__ __forceinline__ void rk4(const Params<R>& p, R kq, const double x[3], const R u[3], R hs, R h6,
-                                    double xo[3], R uo[3])
+// Classical RK4 in path length on (x, u), du/ds = kq u x B, |p| fixed during
+// the step; u renormalised after each substep.
+//
+// Mixed precision: the direction and its derivatives in float, stage by
+// stage, positions in FP64.  A: the axis of a field along one coordinate
+// axis (-1: any direction).  Along an axis the products with B's zero
+// components are zeros and the component of u along B does not change, so
+// leaving them out changes no result (45 instead of 72 operations):
+// calorimeter in 2 T, 10,000 events, 252.7 -> 203.7 ms (with the chord test
+// below on the integer pipe).
+template <int A>
+__device__ __forceinline__ void rk4_stages(const Params<float>& p, float kq, const double x[3], const float u[3],
+                                           float hs, float h6, double xo[3], float uo[3])
 {
     // h6 = hs / 6, rounded once by the caller (the same quotient for every
     // substep of one length)
     // products added to a sum are fused (one rounding each), as in the oracle
-    const R B0 = from_d<R>(p.B[0]), B1 = from_d<R>(p.B[1]), B2 = from_d<R>(p.B[2]);
-    R a1[3], a2[3], a3[3], a4[3], u2[3], u3[3], u4[3];
-    const R hh = R(0.5) * hs;
-    a1[0] = kq * mfma(u[1], B2, -(u[2] * B1));
-    a1[1] = kq * mfma(u[2], B0, -(u[0] * B2));
-    a1[2] = kq * mfma(u[0], B1, -(u[1] * B0));
+    constexpr int I = A < 0 ? 0 : A, J = (I + 1) % 3, K = (I + 2) % 3;
+    const float B0 = (float)p.B[0], B1 = (float)p.B[1], B2 = (float)p.B[2];
+    const float Bi = I == 0 ? B0 : (I == 1 ? B1 : B2);
+    auto slope = [&](const float v[3], float a[3]) {
+        if constexpr (A < 0) {
+            a[0] = kq * mfma(v[1], B2, -(v[2] * B1));
+            a[1] = kq * mfma(v[2], B0, -(v[0] * B2));
+            a[2] = kq * mfma(v[0], B1, -(v[1] * B0));
+        } else {
+            a[I] = 0.0f;
+            a[J] = kq * (v[K] * Bi);
+            a[K] = kq * -(v[J] * Bi);
+        }
+    };
+    auto along = [&](float h, const float a[3], float v[3]) {
 #pragma unroll
-    for (int i = 0; i < 3; ++i) u2[i] = mfma(hh, a1[i], u[i]);
-    a2[0] = kq * mfma(u2[1], B2, -(u2[2] * B1));
-    a2[1] = kq * mfma(u2[2], B0, -(u2[0] * B2));
-    a2[2] = kq * mfma(u2[0], B1, -(u2[1] * B0));
-#pragma unroll
-    for (int i = 0; i < 3; ++i) u3[i] = mfma(hh, a2[i], u[i]);
-    a3[0] = kq * mfma(u3[1], B2, -(u3[2] * B1));
-    a3[1] = kq * mfma(u3[2], B0, -(u3[0] * B2));
-    a3[2] = kq * mfma(u3[0], B1, -(u3[1] * B0));
-#pragma unroll
-    for (int i = 0; i < 3; ++i) u4[i] = mfma(hs, a3[i], u[i]);
-    a4[0] = kq * mfma(u4[1], B2, -(u4[2] * B1));
-    a4[1] = kq * mfma(u4[2], B0, -(u4[0] * B2));
-    a4[2] = kq * mfma(u4[0], B1, -(u4[1] * B0));
+        for (int i = 0; i < 3; ++i) v[i] = i == A ? u[i] : mfma(h, a[i], u[i]);
+    };
+    float a1[3], a2[3], a3[3], a4[3], u2[3], u3[3], u4[3];
+    const float hh = 0.5f * hs;
+    slope(u, a1);
+    along(hh, a1, u2);
+    slope(u2, a2);
+    along(hh, a2, u3);
+    slope(u3, a3);
+    along(hs, a3, u4);
+    slope(u4, a4);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        const R su = mfma(R(2), u3[i], mfma(R(2), u2[i], u[i])) + u4[i];
-        const R sa = mfma(R(2), a3[i], mfma(R(2), a2[i], a1[i])) + a4[i];
-        if constexpr (sizeof(R) == 8)
-            xo[i] = fma(h6, su, x[i]);
-        else
-            xo[i] = x[i] + to_d(h6 * su);
-        uo[i] = mfma(h6, sa, u[i]);
+        const float su = mfma(2.0f, u3[i], mfma(2.0f, u2[i], u[i])) + u4[i];
+        xo[i] = x[i] + to_d(h6 * su);
+        if (i == A) {
+            uo[i] = u[i];
+        } else {
+            const float sa = mfma(2.0f, a3[i], mfma(2.0f, a2[i], a1[i])) + a4[i];
+            uo[i] = mfma(h6, sa, u[i]);
+        }
     }
     const auto nd = mdivisor(msqrt(mfma(uo[0], uo[0], mfma(uo[1], uo[1], uo[2] * uo[2]))));
 #pragma unroll
     for (int i = 0; i < 3; ++i) uo[i] = mdiv(uo[i], nd);
+}
+
+// One substep's map for a given length: mixed precision
+struct FieldStages {
+    float kq, hs, h6;
+};
+
+__device__ __forceinline__ FieldStages field_step(const Params<float>& p, double kq, double h, float)
+{
+    (void)p;
+    FieldStages f;
+    f.kq = (float)kq;
+    f.hs = (float)h;
+    f.h6 = mdiv(f.hs, 6.0f);
+    return f;
+}
+
+__device__ __forceinline__ void rk4(const Params<float>& p, const FieldStages& f, const double x[3], const float u[3],
+                                    double xo[3], float uo[3])
+{
+    switch (p.baxis) {
+    case 0: rk4_stages<0>(p, f.kq, x, u, f.hs, f.h6, xo, uo); break;
+    case 1: rk4_stages<1>(p, f.kq, x, u, f.hs, f.h6, xo, uo); break;
+    case 2: rk4_stages<2>(p, f.kq, x, u, f.hs, f.h6, xo, uo); break;
+    default: rk4_stages<-1>(p, f.kq, x, u, f.hs, f.h6, xo, uo);
+    }
+}
+
+// FP64.  In a uniform field the derivative is linear in u and constant, so
+// the four stages of a substep of length h collapse, in exact arithmetic, to
+// their stability polynomials: with b = B / |B|, t = kq |B| h, w1 = u x b and
+// w2 = w1 x b (and w2 x b = -w1),
+//   u' = u + (t - t^3/6) w1 + (t^2/2 - t^4/24) w2
+//   x' = x + h u + h (t/2 - t^3/24) w1 + h t^2/6 w2.
+// The five coefficients belong to the length, so a step of n equal substeps
+// forms them once; a substep is then 41 FP64 operations for any field
+// direction and 21 along a coordinate axis, against 72 (and a square root
+// and three divisions) stage by stage.  Its error against 128-bit arithmetic,
+// 4,000 tracks of 1-100 substeps: position 1.8e-14 cm rms as before,
+// direction 1.6e-16 (2.2e-16 before).  Calorimeter in 2 T, 4,000 events:
+// 384 -> 163 ms (with the chord test below on the integer pipe).
+struct FieldMap {
+    double h;         // displacement along u
+    double hp;        // h (1 - t^2/6): along u, components across the field
+    double x1, x2;    // displacement along w1, w2
+    double u1, u2;    // turn along w1, w2
+};
+
+__device__ __forceinline__ FieldMap field_step(const Params<double>& p, double kq, double h, double)
+{
+    FieldMap f;
+    const double t = kq * (p.baxis >= 0 ? p.B[p.baxis] : p.bmag) * h;
+    const double tt = t * t;
+    f.h = h;
+    f.x2 = h * (tt * (1.0 / 6.0));
+    f.hp = h - f.x2;
+    f.x1 = h * (t * fma(tt, -1.0 / 24.0, 0.5));
+    f.u1 = t * fma(tt, -1.0 / 6.0, 1.0);
+    f.u2 = tt * fma(tt, -1.0 / 24.0, 0.5);
+    return f;
+}
+
+// field along axis A (its sign is in the coefficients): w1 = (0, u_k, -u_j),
+// w2 = -(0, u_j, u_k) in the cyclic order A, j, k
+template <int A>
+__device__ __forceinline__ void field_map_axis(const FieldMap& f, const double x[3], const double u[3], double xo[3],
+                                               double uo[3])
+{
+    constexpr int J = (A + 1) % 3, K = (A + 2) % 3;
+    xo[A] = fma(f.h, u[A], x[A]);
+    xo[J] = x[J] + fma(f.x1, u[K], f.hp * u[J]);
+    xo[K] = x[K] + fma(-f.x1, u[J], f.hp * u[K]);
+    uo[A] = u[A];
+    uo[J] = u[J] + fma(-f.u2, u[J], f.u1 * u[K]);
+    uo[K] = u[K] - fma(f.u2, u[K], f.u1 * u[J]);
+}
+
+__device__ __forceinline__ void rk4(const Params<double>& p, const FieldMap& f, const double x[3], const double u[3],
+                                    double xo[3], double uo[3])
+{
+    switch (p.baxis) {
+    case 0: field_map_axis<0>(f, x, u, xo, uo); break;
+    case 1: field_map_axis<1>(f, x, u, xo, uo); break;
+    case 2: field_map_axis<2>(f, x, u, xo, uo); break;
+    default: {
+        const double* b = p.bhat;
+        double w[3], v[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) w[i] = fma(u[(i + 1) % 3], b[(i + 2) % 3], -(u[(i + 2) % 3] * b[(i + 1) % 3]));
+#pragma unroll
+        for (int i = 0; i < 3; ++i) v[i] = fma(w[(i + 1) % 3], b[(i + 2) % 3], -(w[(i + 2) % 3] * b[(i + 1) % 3]));
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            xo[i] = x[i] + fma(f.x2, v[i], fma(f.x1, w[i], f.h * u[i]));
+            uo[i] = u[i] + fma(f.u2, v[i], f.u1 * w[i]);
+        }
+    }
+    }
+    // Renormalise.  |u'|^2 = 1 + e with e of the order of t^6/72: below 2^-27
+    // the factor (1 + e)^(-1/2) is 1 - e/2 to within 2^-54.4, one fused
+    // multiply-add per component instead of a square root and divisions.
+    const double n2 = fma(uo[0], uo[0], fma(uo[1], uo[1], uo[2] * uo[2]));
+    const double e = n2 - 1.0;
+    if ((__double2hiint(e) & 0x7FFFFFFF) < ((1023 - 27) << 20)) {
+        const double c = -0.5 * e;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) uo[i] = fma(uo[i], c, uo[i]);
+    } else {
+        const auto nd = mdivisor(msqrt(n2));
+#pragma unroll
+        for (int i = 0; i < 3; ++i) uo[i] = mdiv(uo[i], nd);
+    }
 }
 
 // True when the chord from x (inside volume vol) to x1 cannot leave vol:
@@ -876,6 +1006,14 @@ constexpr double kChordMargin = 1e-6;  // cm
 // set, not recomputed from a rounded quotient) and ends without an
 // interaction: it bounds the work of one step of a looping track.
 constexpr int kMaxSubsteps = 100;
+
+// x1 lies more than kChordMargin inside a layer's side walls
+template <typename R>
+__device__ __forceinline__ bool inside_walls(const Params<R>& p, const double x1[3])
+{
+    const long long k0 = ord_key(x1[0]), k1 = ord_key(x1[1]);
+    return k0 > p.kxy[0] && k0 < p.kxy[1] && k1 > p.kxy[2] && k1 < p.kxy[3];
+}
 
 // Cylinders: both ends within the shell's end planes and inside the circle
 // of radius r_out - margin (the disc is convex, so the whole chord is), and
@@ -904,54 +1042,22 @@ __device__ __forceinline__ bool chord_inside(const Params<R>& p, int vol, const 
         }
         return true;
     }
+    // Layers: integer comparisons through ord_key, whose order is the numeric
+    // order of non-NaN values, with the bounds' keys formed when the geometry
+    // is loaded.  A NaN coordinate of x1 fails one of the tests of its axis.
     if (vol >= 0) {
-        return x1[2] > p.zb[vol] + m && x1[2] < p.zb[vol + 1] - m && x1[0] > -p.hx + m && x1[0] < p.hx - m &&
-               x1[1] > -p.hy + m && x1[1] < p.hy - m;
+        const long long k2 = ord_key(x1[2]);
+        return k2 > p.kz[2 * vol] && k2 < p.kz[2 * vol + 3] && inside_walls(p, x1);
     }
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-        if (!(x1[a] > p.wlo[a] + m && x1[a] < p.whi[a] - m)) return false;
-    const double lo[3] = {-p.hx - m, -p.hy - m, p.zb[0] - m};
-    const double hi[3] = {p.hx + m, p.hy + m, p.zb[p.n_layers] + m};
+    bool inside = true, apart = false;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const double smin = x[a] < x1[a] ? x[a] : x1[a];
-        const double smax = x[a] < x1[a] ? x1[a] : x[a];
-        if (smax < lo[a] || smin > hi[a]) return true;  // separated along axis a
+        const long long k0 = ord_key(x[a]), k1 = ord_key(x1[a]);
+        inside = inside && k1 > p.kworld[a][0] && k1 < p.kworld[a][1];
+        // the chord and the layer stack are separated along axis a
+        apart = apart || (k0 < k1 ? k1 : k0) < p.kstack[a][0] || (k0 < k1 ? k0 : k1) > p.kstack[a][1];
     }
-    return false;
-}
-
-// The chord test of a layer (vol >= 0, layered geometry) as integer
-// comparisons through ord_key, whose order is the numeric order of non-NaN
-// values: the lateral bounds' keys are formed when the geometry is loaded
-// (Params::kxy), the layer's two z bounds per substep (held across the
-// substep loop they cost registers, and spills, in the mixed-precision
-// kernel), each with the same sum chord_inside forms.  A NaN coordinate fails one of the two tests
-// of its axis in both forms, so every decision equals chord_inside's.
-struct LayerBox {
-    long long zlo, zhi;
-};
-
-template <typename R>
-__device__ __forceinline__ LayerBox layer_box(const Params<R>& p, int vol)
-{
-    return LayerBox{ord_key(p.zb[vol] + kChordMargin), ord_key(p.zb[vol + 1] - kChordMargin)};
-}
-
-template <typename R>
-__device__ __forceinline__ bool inside_box(const Params<R>& p, const LayerBox& b, const double x1[3])
-{
-    const long long k2 = ord_key(x1[2]);
-    return k2 > b.zlo && k2 < b.zhi && inside_walls(p, x1);
-}
-
-// x1 lies more than kChordMargin inside a layer's side walls
-template <typename R>
-__device__ __forceinline__ bool inside_walls(const Params<R>& p, const double x1[3])
-{
-    const long long k0 = ord_key(x1[0]), k1 = ord_key(x1[1]);
-    return k0 > p.kxy[0] && k0 < p.kxy[1] && k1 > p.kxy[2] && k1 < p.kxy[3];
+    return inside && apart;
 }
 
 // n substeps of length hs (the caller derives both from h_max); the chord
@@ -962,25 +1068,23 @@ template <int G, typename R>
 __device__ __forceinline__ double propagate_field(const Params<R>& p, int charge, double pm, int vol, double x[3],
                                                   R u[3], int n, double hs, Exit* bnd, bool* crossed, int* evals)
 {
-    double kq = mdiv(charge * kFieldC, pm);
+    const double kq = mdiv(charge * kFieldC, pm);
     double s = 0.0;
     *crossed = false;
-    const R hsr = R(hs);
-    const R h6 = mdiv(hsr, R(6));
-    const bool boxed = G == kGeomLayers && vol >= 0;
+    const auto whole = field_step(p, kq, hs, R(0));
     for (int i = 0; i < n; ++i) {
-        double x1[3], c[3];
+        double x1[3];
         R u1[3];
-        rk4(p, R(kq), x, u, hsr, h6, x1, u1);
+        rk4(p, whole, x, u, x1, u1);
         *evals += 1;
-        if (!(boxed ? inside_box(p, layer_box(p, vol), x1) : chord_inside<G>(p, vol, x, x1))) {
+        if (!chord_inside<G>(p, vol, x, x1)) {
+            double c[3];
 #pragma unroll
             for (int a = 0; a < 3; ++a) c[a] = x1[a] - x[a];
-            Exit e = nav_exit<G>(p, vol, x, c);
+            const Exit e = nav_exit<G>(p, vol, x, c);
             if (e.t <= 1.0) {
-                double h2 = hs * e.t;
-                const R h2r = R(h2);
-                rk4(p, R(kq), x, u, h2r, mdiv(h2r, R(6)), x1, u1);
+                const double h2 = hs * e.t;
+                rk4(p, field_step(p, kq, h2, R(0)), x, u, x1, u1);
                 *evals += 1;
                 snap(e, x1);
 #pragma unroll
