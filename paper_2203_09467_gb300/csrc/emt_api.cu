@@ -769,9 +769,9 @@ emt_status run_loop(emt_ctx* c, int32_t max_iterations, emt_run_stats* st)
         }
         int side = (int)(c->it & 1), cin = (int)(c->it % 3), cout = (int)((c->it + 1) % 3),
             cclr = (int)((c->it + 2) % 3);
-        // the fused step takes block-sized chunks, the transport kernel
-        // warp-sized ones (a block for every warp chunk while blocks last)
-        const int per = c->plan.split && c->opt.max_active <= 0 ? 32 : c->block;
+        // a block for every warp-sized chunk while resident blocks last
+        // (track selection: block-sized chunks)
+        const int per = c->opt.max_active <= 0 ? 32 : c->block;
         int64_t chunks = (c->live_g + per - 1) / per + (c->live_c + per - 1) / per;
         int grid = (int)std::max<int64_t>(1, std::min<int64_t>(chunks, c->resident_blocks[p.has_field]));
         EMT_CUDA(c, cudaEventRecord(c->ev0, c->stream));
@@ -1826,7 +1826,7 @@ extern "C" emt_status emt_transport_static(int32_t device, uint32_t seed, const 
     unsigned long long steps[2] = {0, 0}, last_steps = 0;
     for (int64_t it = 0; live_g + live_c > 0; ++it) {
         const int side = (int)(it & 1), cin = (int)(it % 3), cout = (int)((it + 1) % 3), cclr = (int)((it + 2) % 3);
-        const int64_t chunks = (live_g + block - 1) / block + (live_c + block - 1) / block;
+        const int64_t chunks = (live_g + 31) / 32 + (live_c + 31) / 32;  // warp-sized
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(chunks, resident));
         if (Launch<double>::step(p, side, cin, cout, cclr, grid, block, st) != cudaSuccess) return EMT_ERR_CUDA;
         if (cudaMemcpyAsync(&h_cnt, pool + pl.cnt + sizeof(Counters) * ((it + 1) % 3), sizeof h_cnt,

@@ -352,6 +352,17 @@ __global__ void __launch_bounds__(BS, transport_threads_per_sm<R, F>() / BS)
 // chunks give warps of fewer models.
 constexpr int kInteractRecords = 2;
 
+// Records in one chunk of an interaction phase over n records on `grid`
+// blocks: kInteractRecords * BS, halved while every chunk would still have a
+// block of its own (down to 64), so that few records spread over the SMs.
+template <int BS>
+__device__ __forceinline__ int interact_chunk(int n, int grid)
+{
+    int ch = BS * kInteractRecords;
+    while (ch > 64 && (n + ch / 2 - 1) / (ch / 2) <= grid) ch >>= 1;
+    return ch;
+}
+
 // copy queue record r of `from` to record k of `to`
 template <typename R>
 __device__ __forceinline__ void copy_record(const InterQueue<R>& from, long long r, const InterQueue<R>& to, long long k)
@@ -385,11 +396,11 @@ template <typename R, int BS, bool X, bool kPipe>
 __device__ __forceinline__ void interact_chunks(const Params<R>& p, const Tracks<R>& qi, const Tracks<R>& qo,
                                                 Counters* co, int cin, const InterQueue<R>& iq, int n_int,
                                                 long long spare, bool unlimited, const InterQueue<R>& qnext,
-                                                int* n_next, unsigned* eh, int& s_chunk, int* count, int* offset,
+                                                int* n_next, unsigned* eh, int& s_chunk, int* count,
                                                 unsigned short* perm, StepTally& tally)
 {
-    constexpr int CH = BS * kInteractRecords;
-    const int chunks = (n_int + CH - 1) / CH;
+    const int ch = interact_chunk<BS>(n_int, (int)gridDim.x);
+    const int chunks = (n_int + ch - 1) / ch;
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const unsigned lanes_below = (1u << lane) - 1u;
@@ -401,8 +412,8 @@ __device__ __forceinline__ void interact_chunks(const Params<R>& p, const Tracks
         if (tid == 0) next = (int)gridDim.x + atomicAdd(&p.cnt[cin].work_b, 1);
         if (tid < kNumModels) count[tid] = 0;
         __syncthreads();
-        const long long r0 = (long long)chunk * CH;
-        const int n_here = (int)(n_int - r0 < CH ? n_int - r0 : CH);
+        const long long r0 = (long long)chunk * ch;
+        const int n_here = (int)(n_int - r0 < ch ? n_int - r0 : ch);
         // counting sort of the chunk's records by model
         int model[kInteractRecords], rank[kInteractRecords];
 #pragma unroll
@@ -416,23 +427,18 @@ __device__ __forceinline__ void interact_chunks(const Params<R>& p, const Tracks
             }
         }
         __syncthreads();
-        if (tid == 0) {
-            int acc = 0;
-            for (int k = 0; k < kNumModels; ++k) {
-                offset[k] = acc;
-                acc += count[k];
-            }
-            offset[kNumModels] = acc;
+        const ModelGroups groups(count, lane);
+#pragma unroll
+        for (int j = 0; j < kInteractRecords; ++j) {
+            const int k = groups.place(model[j], rank[j]);
+            if (model[j] >= 0) perm[k] = (unsigned short)(j * BS + tid);
         }
         __syncthreads();
-#pragma unroll
-        for (int j = 0; j < kInteractRecords; ++j)
-            if (model[j] >= 0) perm[offset[model[j]] + rank[j]] = (unsigned short)(j * BS + tid);
-        __syncthreads();
 
-        for (int round = 0; round < kInteractRecords; ++round) {
-            const int pos = round * BS + tid;  // sorted position: a warp takes 32 consecutive ones
-            const bool mine = pos < n_here;
+        for (int round = tid >> 5; round < groups.rounds; round += BS / 32) {
+            int m_round;
+            const int pos = groups.record(round, lane, m_round);
+            const bool mine = pos >= 0;
             TrackReg<R> t;
             Effects fx;
             StepOut<R> o;
@@ -462,7 +468,7 @@ __device__ __forceinline__ void interact_chunks(const Params<R>& p, const Tracks
                 fx.col = score_col(p, t.vol, t.x[2]);
                 fx.finished = false;
                 fx.live_delta = 0;
-                interaction_part<X>(p, t, (int)(tv >> 24), fx, o);
+                interaction_part<X>(p, t, m_round, fx, o);
                 stepped = true;
             }
             if (!unlimited) {
@@ -528,7 +534,6 @@ __global__ void __launch_bounds__(BS, 512 / BS) k_interact(Params<R> p, int side
     constexpr int CH = BS * kInteractRecords;
     __shared__ int s_chunk;
     __shared__ int count[kNumModels];
-    __shared__ int offset[kNumModels + 1];
     __shared__ unsigned short perm[CH];
     __shared__ unsigned s_eh[S ? kEBins : 1];
     constexpr bool select = S;
@@ -540,7 +545,7 @@ __global__ void __launch_bounds__(BS, 512 / BS) k_interact(Params<R> p, int side
     StepTally tally;
     interact_chunks<R, BS, X, false>(p, p.q[side], p.q[side ^ 1], &p.cnt[cout], cin, p.iq, p.cnt[cin].n_int,
                                      p.Q - ntot, 2 * ntot <= p.Q, p.iq, nullptr, select ? s_eh : nullptr, s_chunk,
-                                     count, offset, perm, tally);
+                                     count, perm, tally);
     flush_tally<false>(p, threadIdx.x & 31, tally);
     if constexpr (select) {
         for (int b = threadIdx.x; b < kEBins; b += BS)
@@ -576,7 +581,6 @@ __global__ void __launch_bounds__(BS, pipe_threads_per_sm<R, F>() / BS)
     constexpr int CH = BS * kInteractRecords;
     __shared__ int s_chunk;
     __shared__ int count[kNumModels];
-    __shared__ int offset[kNumModels + 1];
     __shared__ unsigned short perm[CH];
     if (blockIdx.x == 0) clear_counters(&p.cnt[cclr]);
     const Tracks<R> qi = p.q[side];
@@ -594,7 +598,7 @@ __global__ void __launch_bounds__(BS, pipe_threads_per_sm<R, F>() / BS)
     // interactions of the previous iteration
     StepTally tally;
     interact_chunks<R, BS, X, true>(p, qi, qo, co, cin, q_prev, n_prev, Q - ntot, 2 * ntot <= Q, q_next, n_next,
-                                    nullptr, s_chunk, count, offset, perm, tally);
+                                    nullptr, s_chunk, count, perm, tally);
 
     // transport of this iteration's tracks (charged first in a field, in
     // the order of k_sort_order)
@@ -605,7 +609,8 @@ __global__ void __launch_bounds__(BS, pipe_threads_per_sm<R, F>() / BS)
     // The first chunk of a warp is fixed, as in k_transport, starting with
     // the blocks that had no interactions to sample.
     const int grid = (int)gridDim.x;
-    const int busy = min((n_prev + CH - 1) / CH, grid);
+    const int ch = interact_chunk<BS>(n_prev, grid);
+    const int busy = min((n_prev + ch - 1) / ch, grid);
     const int warps = grid * (BS / 32);
     int chunk = ((int)blockIdx.x < busy ? (int)blockIdx.x + grid - busy : (int)blockIdx.x - busy) +
                 grid * (int)(threadIdx.x >> 5);

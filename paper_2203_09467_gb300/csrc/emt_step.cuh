@@ -716,9 +716,52 @@ struct Staging {
     uint32_t ev[BS];
     uint32_t step[BS];
     uint32_t tv[BS];
-    unsigned char model[BS];
     int count[kNumModels];
-    int offset[kNumModels + 1];
+};
+
+// The records of a block's chunk grouped by model, and the rounds in which
+// warps sample them: each model's records start a new round, so a round of 32
+// records runs one sampler.  A warp that holds several models runs their
+// samplers one after the other; with a round of its own each model of a
+// small chunk is sampled by another warp at the same time.  Every warp forms
+// the groups from the shared counts on its own (lane m holds model m).  With
+// chunks that shrink to the population (below, and interact_chunk): one
+// 10 GeV event 4.09 -> 3.33 ms, 1,000 x 100 MeV into the slab 1.22 -> 0.99 ms,
+// FP64 calorimeter of 10,000 events 43.0 -> 39.4 ms, mixed 22.2 ms as before.
+struct ModelGroups {
+    int count, first;          // records of the lane's model, records before it
+    int rounds_end;            // rounds up to and including the lane's model
+    int rounds;                // rounds of the chunk
+
+    __device__ __forceinline__ ModelGroups(const int* counts, int lane)
+    {
+        static_assert(kNumModels <= 32, "one lane per model");
+        count = lane < kNumModels ? counts[lane] : 0;
+        const int mine = (count + 31) >> 5;
+        int c = count | (mine << 16);  // a chunk holds fewer than 2^16 records
+#pragma unroll
+        for (int d = 1; d < kNumModels; d <<= 1) {
+            const int y = __shfl_up_sync(0xFFFFFFFFu, c, d);
+            if (lane >= d) c += y;
+        }
+        first = (c & 0xFFFF) - count;
+        rounds_end = c >> 16;
+        rounds = __shfl_sync(0xFFFFFFFFu, rounds_end, kNumModels - 1);
+    }
+    // place of record `rank` of model m in model order (every lane calls it)
+    __device__ __forceinline__ int place(int m, int rank) const
+    {
+        return __shfl_sync(0xFFFFFFFFu, first, m & (kNumModels - 1)) + rank;
+    }
+    // the lane's record (in model order) in round r, -1 if none, and the model
+    __device__ __forceinline__ int record(int r, int lane, int& model) const
+    {
+        model = __popc(__ballot_sync(0xFFFFFFFFu, lane < kNumModels && rounds_end <= r));
+        const int n = __shfl_sync(0xFFFFFFFFu, count, model);
+        const int i = (r - __shfl_sync(0xFFFFFFFFu, rounds_end, model) + ((n + 31) >> 5)) * 32 + lane;
+        const int f = __shfl_sync(0xFFFFFFFFu, first, model);
+        return i < n ? f + i : -1;
+    }
 };
 
 
@@ -747,7 +790,12 @@ __device__ __forceinline__ void step_body(const Params<R>& p, int side, int cin,
     const long long ntot = (long long)nG + nC;
     const long long spare = Q - ntot;
     const bool unlimited = 2 * ntot <= Q;
-    const int bs = BS;
+    // tracks per chunk: the block size, halved (down to one warp) while the
+    // blocks of the grid would not all get a chunk; a step of few tracks
+    // lasts as long as its dependent chain, which spread-out warps do not
+    // share an SM's FP64 pipe for
+    int bs = BS;
+    while (bs > 32 && (nG + bs / 2 - 1) / (bs / 2) + (nC + bs / 2 - 1) / (bs / 2) <= (int)gridDim.x) bs >>= 1;
     const int chunksG = (nG + bs - 1) / bs;
     const int chunksC = (nC + bs - 1) / bs;
     const int tid = threadIdx.x;
@@ -767,7 +815,7 @@ __device__ __forceinline__ void step_body(const Params<R>& p, int side, int cin,
         const bool photon_chunk = chunk < chunksG;
         const long long i = photon_chunk ? (long long)chunk * bs + tid : (long long)(chunk - chunksG) * bs + tid;
         const long long n_here = photon_chunk ? nG : nC;
-        const bool active = i < n_here;
+        const bool active = tid < bs && i < n_here;
         const long long src = photon_chunk ? i : Q - nC + i;
 
         // ---- phase A: own track
@@ -794,17 +842,9 @@ __device__ __forceinline__ void step_body(const Params<R>& p, int side, int cin,
         emit<1>(p, qo, co, lane, o, t.x, t.ev, t.vol);
         report_finished(p, t.ev, live);
         __syncthreads();
-        if (tid == 0) {
-            int acc = 0;
-            for (int m = 0; m < kNumModels; ++m) {
-                sg.offset[m] = acc;
-                acc += sg.count[m];
-            }
-            sg.offset[kNumModels] = acc;
-        }
-        __syncthreads();
+        const ModelGroups groups(sg.count, lane);
+        const int k = groups.place(model, rank);
         if (model != kNoInteraction) {
-            const int k = sg.offset[model] + rank;
             sg.x[0][k] = t.x[0];
             sg.x[1][k] = t.x[1];
             sg.x[2][k] = t.x[2];
@@ -818,68 +858,70 @@ __device__ __forceinline__ void step_body(const Params<R>& p, int side, int cin,
             sg.ev[k] = t.ev;
             sg.step[k] = t.step;
             sg.tv[k] = pack_tv(t.type, t.vol);
-            sg.model[k] = (unsigned char)model;
         }
         __syncthreads();
 
-        // ---- phase B: sampled interactions, sorted by model
-        const int n_int = sg.offset[kNumModels];
-        bool mine = tid < n_int;
-        o.n = 0;
-        bool stepped = false;
-        long long rsrc = 0;
-        if (mine) {
-            t.x[0] = sg.x[0][tid];
-            t.x[1] = sg.x[1][tid];
-            t.x[2] = sg.x[2][tid];
-            t.u[0] = sg.u[0][tid];
-            t.u[1] = sg.u[1][tid];
-            t.u[2] = sg.u[2][tid];
-            t.T = sg.T[tid];
-            t.uid = sg.uid[tid];
-            t.ev = sg.ev[tid];
-            t.step = sg.step[tid];
-            t.type = tv_type(sg.tv[tid]);
-            t.vol = tv_vol(sg.tv[tid]);
-            rsrc = sg.src[tid];
-            fx.dep = sg.dep[tid];
-            fx.esc = 0.0;
-            fx.kill = 0.0;
-            fx.col = score_col(p, t.vol, t.x[2]);
-            fx.finished = false;
-            fx.live_delta = 0;
-            interaction_part<X>(p, t, (int)sg.model[tid], fx, o);
-            stepped = true;
-        }
-        if (!unlimited) {
-            const bool need = stepped && o.n == 2;
-            const unsigned m = __ballot_sync(0xFFFFFFFFu, need);
-            if (m) {
-                const int k = __popc(m);
-                const int leader = __ffs(m) - 1;
-                int got = 0;
-                if (lane == leader) {
-                    int old = atomicAdd(&p.cnt[cin].used, k);
-                    long long avail = spare - old;
-                    got = avail <= 0 ? 0 : (avail >= k ? k : (int)avail);
-                    if (got < k) atomicSub(&p.cnt[cin].used, k - got);
-                }
-                got = __shfl_sync(0xFFFFFFFFu, got, leader);
-                if (need && __popc(m & lanes_below) >= got) {
-                    // no room for the second output: discard the whole step
-                    load_track(qi, rsrc, t);
-                    copy_out(t, o);
-                    stepped = false;
+        // ---- phase B: sampled interactions, a round of one model per warp
+        for (int round = tid >> 5; round < groups.rounds; round += BS / 32) {
+            int m;
+            const int r = groups.record(round, lane, m);
+            const bool mine = r >= 0;
+            o.n = 0;
+            bool stepped = false;
+            long long rsrc = 0;
+            if (mine) {
+                t.x[0] = sg.x[0][r];
+                t.x[1] = sg.x[1][r];
+                t.x[2] = sg.x[2][r];
+                t.u[0] = sg.u[0][r];
+                t.u[1] = sg.u[1][r];
+                t.u[2] = sg.u[2][r];
+                t.T = sg.T[r];
+                t.uid = sg.uid[r];
+                t.ev = sg.ev[r];
+                t.step = sg.step[r];
+                t.type = tv_type(sg.tv[r]);
+                t.vol = tv_vol(sg.tv[r]);
+                rsrc = sg.src[r];
+                fx.dep = sg.dep[r];
+                fx.esc = 0.0;
+                fx.kill = 0.0;
+                fx.col = score_col(p, t.vol, t.x[2]);
+                fx.finished = false;
+                fx.live_delta = 0;
+                interaction_part<X>(p, t, m, fx, o);
+                stepped = true;
+            }
+            if (!unlimited) {
+                const bool need = stepped && o.n == 2;
+                const unsigned mt = __ballot_sync(0xFFFFFFFFu, need);
+                if (mt) {
+                    const int k = __popc(mt);
+                    const int leader = __ffs(mt) - 1;
+                    int got = 0;
+                    if (lane == leader) {
+                        int old = atomicAdd(&p.cnt[cin].used, k);
+                        long long avail = spare - old;
+                        got = avail <= 0 ? 0 : (avail >= k ? k : (int)avail);
+                        if (got < k) atomicSub(&p.cnt[cin].used, k - got);
+                    }
+                    got = __shfl_sync(0xFFFFFFFFu, got, leader);
+                    if (need && __popc(mt & lanes_below) >= got) {
+                        // no room for the second output: discard the whole step
+                        load_track(qi, rsrc, t);
+                        copy_out(t, o);
+                        stepped = false;
+                    }
                 }
             }
+            live = 1;
+            if (stepped) live = apply_effects(p, t.ev, t.type, t.step, fx);
+            const int nd = __popc(__ballot_sync(0xFFFFFFFFu, mine && !stepped));
+            tally.steps -= nd;
+            tally.deferred += nd;
+            emit<2>(p, qo, co, lane, o, t.x, t.ev, t.vol);
+            report_finished(p, t.ev, live);
         }
-        live = 1;
-        if (stepped) live = apply_effects(p, t.ev, t.type, t.step, fx);
-        const int nd = __popc(__ballot_sync(0xFFFFFFFFu, mine && !stepped));
-        tally.steps -= nd;
-        tally.deferred += nd;
-        emit<2>(p, qo, co, lane, o, t.x, t.ev, t.vol);
-        report_finished(p, t.ev, live);
         if (tid == 0) s_chunk = next;
         __syncthreads();
         chunk = s_chunk;
