@@ -138,11 +138,11 @@ __device__ __forceinline__ int apply_effects(const Params<R>& p, uint32_t ev, in
     return live;
 }
 
-// Track-steps taken and deferred by a warp (the same in every lane) and RK4
-// evaluations of each lane, kept in registers and added to the run's totals
-// once per kernel.
+// Track-steps taken, deferred and held back by a warp (the same in every
+// lane) and RK4 evaluations of each lane, kept in registers and added to the
+// run's totals once per kernel.
 struct StepTally {
-    int steps = 0, deferred = 0;
+    int steps = 0, deferred = 0, held = 0;
     unsigned substeps = 0;
 };
 
@@ -154,6 +154,7 @@ __device__ __forceinline__ void flush_tally(const Params<R>& p, int lane, const 
     if (lane != 0) return;
     if (c.steps) atomicAdd(&p.total_steps[0], (unsigned long long)(long long)c.steps);
     if (c.deferred) atomicAdd(&p.total_steps[1], (unsigned long long)c.deferred);
+    if (c.held) atomicAdd(&p.total_steps[2], (unsigned long long)c.held);
     if (sub) atomicAdd(&p.total_steps[3], (unsigned long long)sub);
 }
 
@@ -195,7 +196,9 @@ __device__ __forceinline__ int transport_part(const Params<R>& p, TrackReg<R>& t
     const R* tab = p.tab + row;
     const R* dtab = p.dtab + row;
 
-    R sig[4] = {R(0), R(0), R(0), R(0)};
+    // cumulative cross sections in the order of the processes: cum[i] is the
+    // sum of the first i + 1, the last of them the total
+    R cum[4] = {R(0), R(0), R(0), R(0)};
     R sig_tot = R(0);
     R Rng = R(0);
     Lookup<R> lk;
@@ -204,18 +207,11 @@ __device__ __forceinline__ int transport_part(const Params<R>& p, TrackReg<R>& t
     lk.clamp = -1;
     if (matter) {
         lk = locate_energy(p, t.T);
-        sig[0] = xs_value(p, tab, dtab, lk, 0);
-        sig[1] = xs_value(p, tab, dtab, lk, 1);
-        sig_tot = sig[0] + sig[1];
-        if (nproc >= 3) {
-            sig[2] = xs_value(p, tab, dtab, lk, 2);
-            sig_tot = sig_tot + sig[2];
-        }
+        cum[0] = xs_value(p, tab, dtab, lk, 0);
+        cum[1] = sig_tot = cum[0] + xs_value(p, tab, dtab, lk, 1);
+        if (nproc >= 3) cum[2] = sig_tot = sig_tot + xs_value(p, tab, dtab, lk, 2);
         if constexpr (X) {
-            if (nproc == 4) {
-                sig[3] = xs_value(p, tab, dtab, lk, 3);
-                sig_tot = sig_tot + sig[3];
-            }
+            if (nproc == 4) cum[3] = sig_tot = sig_tot + xs_value(p, tab, dtab, lk, 3);
         }
     }
     const R kInf = R(__longlong_as_double(0x7FF0000000000000ll));
@@ -230,18 +226,11 @@ __device__ __forceinline__ int transport_part(const Params<R>& p, TrackReg<R>& t
         // interacts (unused otherwise); taking it here frees the cross
         // sections and the draw state before the propagation.
         const R xsel = draw<R>(dr) * sig_tot;
-        R c = R(0);
-        bool open = true;
+        // the first process whose cumulative sum exceeds xsel (the last one
+        // if rounding leaves none)
 #pragma unroll
-        for (int i = 0; i < (X ? 4 : 3); ++i) {
-            if (open && i < nproc) {
-                c += sig[i];
-                if (lt_pos(xsel, c)) {
-                    proc = i;
-                    open = false;
-                }
-            }
-        }
+        for (int i = (X ? 2 : 1); i >= 0; --i)
+            if (i < nproc - 1 && lt_pos(xsel, cum[i])) proc = i;
     }
     R s_max = kInf;
     if (charged && matter) {
@@ -301,7 +290,7 @@ __device__ __forceinline__ int transport_part(const Params<R>& p, TrackReg<R>& t
                 const bool up = gt_zero(ud[2]);
                 const double pl = p.zb[t.vol + (up ? 1 : 0)];
                 double te = mdiv(pl - t.x[2], ud[2]);
-                if (te < 0.0) te = 0.0;
+                if (__double_as_longlong(te) < 0) te = 0.0;
                 boundary = le_pos(te, s_physd);
                 s = boundary ? te : s_physd;
                 double x1[3];
@@ -387,16 +376,16 @@ __device__ __forceinline__ int transport_part(const Params<R>& p, TrackReg<R>& t
     // 9: the model chosen above, and channels closed at the post-loss energy
     const R T = t.T;
     if (t.type == 0) {
-        if (proc == 0) return T > from_d<R>(p.bk[mi]) ? kPhoto : kNoInteraction;
+        if (proc == 0) return lt_pos(from_d<R>(p.bk[mi]), T) ? kPhoto : kNoInteraction;
         if (proc == 1) return kCompton;
         if (X && proc == 3) return kRayleigh;
-        return T > R(2.0 * kMe) ? kPair : kNoInteraction;
+        return lt_pos(R(2.0 * kMe), T) ? kPair : kNoInteraction;
     }
     if (proc == 0) {
-        if (t.type == 1) return T > R(2) * pcut(p, 1) ? kMoller : kNoInteraction;
-        return T > pcut(p, 1) ? kBhabha : kNoInteraction;
+        if (t.type == 1) return lt_pos(R(2) * pcut(p, 1), T) ? kMoller : kNoInteraction;
+        return lt_pos(pcut(p, 1), T) ? kBhabha : kNoInteraction;
     }
-    if (proc == 1) return T > pcut(p, 0) ? kBrems : kNoInteraction;
+    if (proc == 1) return lt_pos(pcut(p, 0), T) ? kBrems : kNoInteraction;
     return kAnnih;
 }
 
