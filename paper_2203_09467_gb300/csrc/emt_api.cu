@@ -559,12 +559,12 @@ emt_status sync_status(emt_ctx* c, const char* where)
 
 // kernel launches of one step: the fused kernel; or the transport and
 // interaction kernels, plus the two sorting launches of the charged tracks
-// in a field (without track selection)
+// in a field
 template <typename R>
 int launches_per_step(const emt_ctx* c, const Params<R>& p)
 {
     if (!c->plan.split) return 1;
-    const int sort = (p.has_field && p.max_active <= 0) ? 2 : 0;
+    const int sort = p.has_field ? 2 : 0;
     return (c->plan.pipelined ? 1 : 2) + sort;
 }
 
@@ -770,9 +770,7 @@ emt_status run_loop(emt_ctx* c, int32_t max_iterations, emt_run_stats* st)
         int side = (int)(c->it & 1), cin = (int)(c->it % 3), cout = (int)((c->it + 1) % 3),
             cclr = (int)((c->it + 2) % 3);
         // a block for every warp-sized chunk while resident blocks last
-        // (track selection: block-sized chunks)
-        const int per = c->opt.max_active <= 0 ? 32 : c->block;
-        int64_t chunks = (c->live_g + per - 1) / per + (c->live_c + per - 1) / per;
+        int64_t chunks = (c->live_g + 31) / 32 + (c->live_c + 31) / 32;
         int grid = (int)std::max<int64_t>(1, std::min<int64_t>(chunks, c->resident_blocks[p.has_field]));
         EMT_CUDA(c, cudaEventRecord(c->ev0, c->stream));
         cudaError_t e =

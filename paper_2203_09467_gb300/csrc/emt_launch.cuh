@@ -170,7 +170,7 @@ static cudaError_t launch_split(const Params<R>& p, int side, int cin, int cout,
 {
     return with_block(block, [&](auto bs) {
         return with_variant(p, [&](auto g, auto f, auto x) {
-            if (!S && f.value) launch_sort(p, side, cin, grid_b, st);
+            if (f.value) launch_sort(p, side, cin, grid_b, st);
             k_transport<R, bs.value, g.value, f.value, S, x.value>
                 <<<grid_a, bs.value, 0, st>>>(p, side, cin, cout, cclr);
             k_interact<R, bs.value, S, x.value><<<grid_b, bs.value, 0, st>>>(p, side, cin, cout);

@@ -195,7 +195,6 @@ template <typename R, int BS, int G, bool F, bool S, bool X>
 __global__ void __launch_bounds__(BS, transport_threads_per_sm<R, F>() / BS)
     k_transport(Params<R> p, int side, int cin, int cout, int cclr)
 {
-    __shared__ int s_chunk;
     __shared__ unsigned s_eh[S ? kEBins : 1];
     __shared__ Selection s_sel, s_spill;
     constexpr bool select = S;
@@ -214,41 +213,7 @@ __global__ void __launch_bounds__(BS, transport_threads_per_sm<R, F>() / BS)
     // the end of the launch instead of the expensive charged work.
     constexpr bool charged_first = F;
 
-    if constexpr (!select) {
-        // Chunks of one warp, taken by each warp on its own (no block
-        // barrier: a warp never waits for the slowest warp of its block).
-        // In a field the charged tracks are taken in the order of
-        // k_sort_order (most expensive first).
-        const int chunksG = (nG + 31) >> 5;
-        const int chunksC = (nC + 31) >> 5;
-        StepTally tally;
-        // The first chunk of a warp is fixed: warp 0 of every block before
-        // warp 1 of any, so that the first (in a field: the most expensive)
-        // chunks run on different SMs.  Later chunks come from the
-        // dispenser, whose answer is on its way during the current chunk.
-        const int warps = (int)gridDim.x * (BS / 32);
-        int chunk = (int)blockIdx.x + (int)gridDim.x * (tid >> 5);
-        while (chunk < chunksG + chunksC) {
-            int next = 0;
-            if (lane == 0) next = warps + atomicAdd(&p.cnt[cin].work, 1);
-            const bool photon_chunk = charged_first ? chunk >= chunksC : chunk < chunksG;
-            const int local = photon_chunk ? (charged_first ? chunk - chunksC : chunk)
-                                           : (charged_first ? chunk : chunk - chunksG);
-            long long i = (long long)local * 32 + lane;
-            const bool active = i < (photon_chunk ? nG : nC);
-            if (charged_first && !photon_chunk && active) i = p.sperm[i];
-            const long long src = photon_chunk ? i : Q - nC + i;
-            TrackReg<R> t;
-            if (active) load_track(qi, src, t);
-            transport_lane<G, F, X>(p, qo, co, p.iq, &p.cnt[cin].n_int, true, lane, t, active, false, src, nullptr,
-                                 tally);
-            chunk = __shfl_sync(0xFFFFFFFFu, next, 0);
-        }
-        flush_tally<F>(p, lane, tally);
-        return;
-    }
-
-    // track selection: chunks of a block (the selection is block-wide)
+    // track selection: the block works out the step's thresholds once
     if constexpr (select) {
         for (int b = threadIdx.x; b < kEBins; b += BS) {
             s_eh[b] = 0u;
@@ -270,21 +235,27 @@ __global__ void __launch_bounds__(BS, transport_threads_per_sm<R, F>() / BS)
         }
         __syncthreads();
     }
-    const int chunksG = (nG + BS - 1) / BS;
-    const int chunksC = (nC + BS - 1) / BS;
+    // Chunks of one warp, taken by each warp on its own (no block barrier: a
+    // warp never waits for the slowest warp of its block).  In a field the
+    // charged tracks are taken in the order of k_sort_order (most expensive
+    // first).  The first chunk of a warp is fixed: warp 0 of every block
+    // before warp 1 of any, so that the first (in a field: the most
+    // expensive) chunks run on different SMs.  Later chunks come from the
+    // dispenser, whose answer is on its way during the current chunk.
+    const int chunksG = (nG + 31) >> 5;
+    const int chunksC = (nC + 31) >> 5;
     StepTally tally;
-    for (;;) {
-        if (tid == 0) s_chunk = atomicAdd(&p.cnt[cin].work, 1);
-        __syncthreads();
-        const int chunk = s_chunk;
-        __syncthreads();
-        if (chunk >= chunksG + chunksC) break;
+    const int warps = (int)gridDim.x * (BS / 32);
+    int chunk = (int)blockIdx.x + (int)gridDim.x * (tid >> 5);
+    while (chunk < chunksG + chunksC) {
+        int next = 0;
+        if (lane == 0) next = warps + atomicAdd(&p.cnt[cin].work, 1);
         const bool photon_chunk = charged_first ? chunk >= chunksC : chunk < chunksG;
         const int local = photon_chunk ? (charged_first ? chunk - chunksC : chunk)
                                        : (charged_first ? chunk : chunk - chunksG);
-        const long long i = (long long)local * BS + tid;
-        const long long n_here = photon_chunk ? nG : nC;
-        bool active = i < n_here;
+        long long i = (long long)local * 32 + lane;
+        bool active = i < (photon_chunk ? nG : nC);
+        if (charged_first && !photon_chunk && active) i = p.sperm[i];
         const long long src = photon_chunk ? i : Q - nC + i;
 
         TrackReg<R> t;
@@ -333,10 +304,11 @@ __global__ void __launch_bounds__(BS, transport_threads_per_sm<R, F>() / BS)
                     }
                 }
             }
-            const unsigned mh = __ballot_sync(0xFFFFFFFFu, held);
-            if (lane == 0 && mh) atomicAdd(&p.total_steps[2], (unsigned long long)__popc(mh));
+            tally.held += __popc(__ballot_sync(0xFFFFFFFFu, held));
         }
-        transport_lane<G, F, X>(p, qo, co, p.iq, &p.cnt[cin].n_int, true, lane, t, active, held, src, s_eh, tally);
+        transport_lane<G, F, X>(p, qo, co, p.iq, &p.cnt[cin].n_int, true, lane, t, active, held, src,
+                                select ? s_eh : nullptr, tally);
+        chunk = __shfl_sync(0xFFFFFFFFu, next, 0);
     }
     flush_tally<F>(p, lane, tally);
     if constexpr (select) {
