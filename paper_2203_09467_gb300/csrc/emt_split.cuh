@@ -500,8 +500,18 @@ __device__ __forceinline__ void interact_chunks(const Params<R>& p, const Tracks
     }
 }
 
+// Resident threads per SM of the interaction kernel (its register budget):
+// FP64 512 (at 768 the shells lose 3.2% and the run with every option 7%),
+// mixed 768 (against 512: calorimeter of 10,000 events 21.8 -> 21.6 ms, in 2 T
+// 203.8 -> 201.1 ms).
+template <typename R>
+constexpr int interact_threads_per_sm()
+{
+    return sizeof(R) == 8 ? 512 : 768;
+}
+
 template <typename R, int BS, bool S, bool X>
-__global__ void __launch_bounds__(BS, 512 / BS) k_interact(Params<R> p, int side, int cin, int cout)
+__global__ void __launch_bounds__(BS, interact_threads_per_sm<R>() / BS) k_interact(Params<R> p, int side, int cin, int cout)
 {
     constexpr int CH = BS * kInteractRecords;
     __shared__ int s_chunk;
