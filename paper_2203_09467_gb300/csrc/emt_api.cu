@@ -109,7 +109,7 @@ Plan make_plan(const emt_options& o)
     p.ray_a = p.add(kMaxMat * sizeof(double));
     p.scratch = p.add((32 + (size_t)kMaxMat * 2 * kMaxGrid) * sizeof(double));
     p.zb = p.add((kMaxLayers + 1) * sizeof(double));
-    p.kz = p.add((kMaxLayers + 1) * 2 * sizeof(long long));
+    p.kz = p.add(kMaxLayers * sizeof(int2));
     p.lmat = p.add(kMaxLayers * sizeof(int));
     p.lbin = p.add(kMaxLayers * sizeof(int));
     const size_t P = (size_t)p.max_prim;
@@ -180,9 +180,9 @@ bool valid_options(const emt_options& o, std::string& why)
 
 // Validate a geometry description and lay out its arrays: zb[n + 1] (plane
 // positions or shell radii), lm[n] (materials), lb[n] (score bins), and the
-// chord test's keys kz[n + 1][2] of the planes.  Returns an error message, or nullptr.
+// chord test's keys kz[n] of the planes.  Returns an error message, or nullptr.
 const char* check_geometry(const emt_layer* layers, int n, const emt_world* w, int n_mat, int max_bins, double* zb,
-                           int* lm, int* lb, long long* kz)
+                           int* lm, int* lb, int2* kz)
 {
     if (n < 1 || n > kMaxLayers) return "layer count out of [1, 4096]";
     if (w->n_bins < 1 || w->n_bins > max_bins) return "n_bins out of [1, max_bins]";
@@ -198,10 +198,7 @@ const char* check_geometry(const emt_layer* layers, int n, const emt_world* w, i
         lm[i] = layers[i].material;
         lb[i] = layers[i].score_bin;
     }
-    for (int i = 0; i <= n; ++i) {
-        kz[2 * i + 0] = ord_key(zb[i] + kChordMargin);
-        kz[2 * i + 1] = ord_key(zb[i] - kChordMargin);
-    }
+    for (int i = 0; i < n; ++i) kz[i] = make_int2(ord_key(zb[i] + kChordMargin), ord_key(zb[i + 1] - kChordMargin));
     if (w->geometry == EMT_GEOM_LAYERS) {
         if (!(w->half_x_cm > 0.0) || !(w->half_y_cm > 0.0)) return "stack half widths";
         const double lo[3] = {-w->half_x_cm, -w->half_y_cm, zb[0]};
@@ -433,7 +430,7 @@ void fill_common(emt_ctx* c, Params<R>& p)
     p.x0 = c->at<double>(pl.x0);
     p.ray_a = c->at<double>(pl.ray_a);
     p.zb = c->at<double>(pl.zb);
-    p.kz = c->at<long long>(pl.kz);
+    p.kz = c->at<int2>(pl.kz);
     p.lmat = c->at<int>(pl.lmat);
     p.lbin = c->at<int>(pl.lbin);
     p.step_bins = pl.step_bins;
@@ -1213,7 +1210,7 @@ emt_status emt_load_geometry(emt_ctx* c, const emt_layer* layers, int32_t n, con
     if (n < 1 || n > kMaxLayers) return fail(c, EMT_ERR_INVALID_ARG, "layer count out of [1, 4096]");
     std::vector<double> zb(n + 1);
     std::vector<int> lm(n), lb(n);
-    std::vector<long long> kz(2 * (size_t)n + 2);
+    std::vector<int2> kz(n);
     if (const char* why =
             check_geometry(layers, n, w, c->n_mat, c->opt.max_bins, zb.data(), lm.data(), lb.data(), kz.data()))
         return fail(c, EMT_ERR_INVALID_ARG, why);
@@ -1222,7 +1219,7 @@ emt_status emt_load_geometry(emt_ctx* c, const emt_layer* layers, int32_t n, con
     EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.zb, zb.data(), sizeof(double) * (n + 1), cudaMemcpyHostToDevice, c->stream));
     EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.lmat, lm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, c->stream));
     EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.lbin, lb.data(), sizeof(int) * n, cudaMemcpyHostToDevice, c->stream));
-    EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.kz, kz.data(), sizeof(long long) * kz.size(), cudaMemcpyHostToDevice, c->stream));
+    EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.kz, kz.data(), sizeof(int2) * kz.size(), cudaMemcpyHostToDevice, c->stream));
     EMT_CUDA(c, cudaStreamSynchronize(c->stream));
     set_geometry(c->pd, n, w, zb.data());
     set_geometry(c->pf, n, w, zb.data());
@@ -1762,10 +1759,10 @@ extern "C" emt_status emt_transport_static(int32_t device, uint32_t seed, const 
     // ---- geometry
     double zb[kMaxLayers + 1];
     int lm[kMaxLayers], lb[kMaxLayers];
-    long long kz[2 * (kMaxLayers + 1)];
+    int2 kz[kMaxLayers];
     if (check_geometry(layers, n_layers, w, n_mat, EMT_STATIC_MAX_BINS, zb, lm, lb, kz)) return EMT_ERR_INVALID_ARG;
     if (cudaMemcpyAsync(pool + pl.zb, zb, sizeof(double) * (n_layers + 1), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(pool + pl.kz, kz, sizeof(long long) * 2 * (n_layers + 1), cudaMemcpyHostToDevice, st) !=
+        cudaMemcpyAsync(pool + pl.kz, kz, sizeof(int2) * n_layers, cudaMemcpyHostToDevice, st) !=
             cudaSuccess ||
         cudaMemcpyAsync(pool + pl.lmat, lm, sizeof(int) * n_layers, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(pool + pl.lbin, lb, sizeof(int) * n_layers, cudaMemcpyHostToDevice, st) != cudaSuccess)

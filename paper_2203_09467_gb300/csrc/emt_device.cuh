@@ -17,6 +17,7 @@
 
 #include "emt_intdiv.cuh"
 #include "emt_intlog.cuh"
+#include "emt_unit.cuh"
 
 namespace emt {
 
@@ -240,11 +241,11 @@ struct Params {
     double hx, hy;
     // ord_key of the bounds of the chord tests, formed once when the geometry
     // is loaded (m = kChordMargin): a layer's side walls -hx + m, hx - m,
-    // -hy + m, hy - m and planes zb[i] + m, zb[i] - m ([n_layers + 1][2]); the
+    // -hy + m, hy - m and its planes zb[i] + m, zb[i + 1] - m ([n_layers]); the
     // world box shrunk by m and the layer stack grown by it, [axis][low, high]
-    long long kxy[4];
-    const long long* kz;
-    long long kworld[3][2], kstack[3][2];
+    int kxy[4];
+    const int2* kz;
+    int kworld[3][2], kstack[3][2];
     double wlo[3], whi[3];
     double B[3];
     double bmag;
@@ -456,20 +457,21 @@ __device__ __forceinline__ bool lt_pos(float a, float b) { return a < b; }
 __device__ __forceinline__ bool gt_zero(double a) { return __double_as_longlong(a) > 0; }
 __device__ __forceinline__ bool gt_zero(float a) { return a > 0.0f; }
 __device__ __forceinline__ bool nonzero(double a) { return ((unsigned long long)__double_as_longlong(a) << 1) != 0ull; }
-// An integer key whose signed order is the numeric order of any two
-// non-NaN doubles of either sign: the magnitude bits, negated for a
-// negative value (so -0 and +0 both map to 0).  A NaN maps beyond every
+// An integer key of a double, monotonic in its value: the high word (sign,
+// exponent and 20 bits of the significand), its magnitude bits inverted for a
+// negative value.  Where the keys of two non-NaN values differ their numeric
+// order is the keys' order; equal keys say nothing.  A NaN maps beyond every
 // finite value on its sign's side.
-__host__ __device__ __forceinline__ long long ord_key(double a)
+__host__ __device__ __forceinline__ int ord_key(double a)
 {
 #ifdef __CUDA_ARCH__
-    const long long b = __double_as_longlong(a);
+    const int h = __double2hiint(a);
 #else
     long long b;
     memcpy(&b, &a, sizeof b);
+    const int h = (int)(b >> 32);
 #endif
-    const long long m = b & 0x7fffffffffffffffll;
-    return b < 0 ? -m : m;
+    return h ^ ((h >> 31) & 0x7fffffff);
 }
 
 // node n with grid[n] <= E < grid[n+1], clamped to [0, n_grid-2]: the FP32
@@ -828,7 +830,8 @@ __device__ __forceinline__ Exit nav_exit(const Params<R>& p, int vol, const doub
 // components are zeros and the component of u along B does not change, so
 // leaving them out changes no result (45 instead of 72 operations):
 // calorimeter in 2 T, 10,000 events, 252.7 -> 203.7 ms (with the chord test
-// below on the integer pipe).
+// below on the integer pipe), and 201.0 -> 162.6 ms with its 32-bit keys and
+// the division by a length near 1 (emt_unit.cuh).
 template <int A>
 __device__ __forceinline__ void rk4_stages(const Params<float>& p, float kq, const double x[3], const float u[3],
                                            float hs, float h6, double xo[3], float uo[3])
@@ -874,9 +877,14 @@ __device__ __forceinline__ void rk4_stages(const Params<float>& p, float kq, con
             uo[i] = mfma(h6, sa, u[i]);
         }
     }
-    const auto nd = mdivisor(msqrt(mfma(uo[0], uo[0], mfma(uo[1], uo[1], uo[2] * uo[2]))));
+    const float s = mfma(uo[0], uo[0], mfma(uo[1], uo[1], uo[2] * uo[2]));
+    if (unit::near_one(s, uo)) {
+        unit::divide(uo, s, uo);  // the same quotients, cheaper
+    } else {
+        const auto nd = mdivisor(msqrt(s));
 #pragma unroll
-    for (int i = 0; i < 3; ++i) uo[i] = mdiv(uo[i], nd);
+        for (int i = 0; i < 3; ++i) uo[i] = mdiv(uo[i], nd);
+    }
 }
 
 // One substep's map for a given length: mixed precision
@@ -884,7 +892,7 @@ struct FieldStages {
     float kq, hs, h6;
 };
 
-__device__ __forceinline__ FieldStages field_step(const Params<float>& p, double kq, double h, float)
+__device__ __forceinline__ FieldStages field_step(const Params<float>& p, double kq, double h, const float*)
 {
     (void)p;
     FieldStages f;
@@ -894,8 +902,8 @@ __device__ __forceinline__ FieldStages field_step(const Params<float>& p, double
     return f;
 }
 
-__device__ __forceinline__ void rk4(const Params<float>& p, const FieldStages& f, const double x[3], const float u[3],
-                                    double xo[3], float uo[3])
+__device__ __forceinline__ void rk4(const Params<float>& p, const FieldStages& f, double, const double x[3],
+                                    const float u[3], double xo[3], float uo[3])
 {
     switch (p.baxis) {
     case 0: rk4_stages<0>(p, f.kq, x, u, f.hs, f.h6, xo, uo); break;
@@ -905,30 +913,50 @@ __device__ __forceinline__ void rk4(const Params<float>& p, const FieldStages& f
     }
 }
 
+// mixed precision renormalises in every substep
+__device__ __forceinline__ void field_end(const FieldStages&, float[3]) {}
+
 // FP64.  In a uniform field the derivative is linear in u and constant, so
 // the four stages of a substep of length h collapse, in exact arithmetic, to
 // their stability polynomials: with b = B / |B|, t = kq |B| h, w1 = u x b and
 // w2 = w1 x b (and w2 x b = -w1),
 //   u' = u + (t - t^3/6) w1 + (t^2/2 - t^4/24) w2
 //   x' = x + h u + h (t/2 - t^3/24) w1 + h t^2/6 w2.
-// The five coefficients belong to the length, so a step of n equal substeps
-// forms them once; a substep is then 41 FP64 operations for any field
-// direction and 21 along a coordinate axis, against 72 (and a square root
-// and three divisions) stage by stage.  Its error against 128-bit arithmetic,
-// 4,000 tracks of 1-100 substeps: position 1.8e-14 cm rms as before,
-// direction 1.6e-16 (2.2e-16 before).  Calorimeter in 2 T, 4,000 events:
-// 384 -> 163 ms (with the chord test below on the integer pipe).
+// The length of u' follows too: |u'|^2 = 1 + e, e = (t^8/576 - t^6/72) |w1|^2
+// (about 1e-12 in a detector), so u' / |u'| = u' + c u' with the same
+// c = -e/2 for every substep of the step (|w1| changes by c of itself in a
+// substep; e^2 is below 2^-54 for |e| < 2^-27), and the renormalisation goes
+// into the coefficients.  The component along an axis field only grows by c
+// of itself, less than a rounding unit: it is formed from the path s since
+// the start of the step, u + s (c/h) u, so that the growth is not lost
+// substep by substep.  What rounding adds to the length, a unit or so in a
+// hundred substeps, is taken off once at the end of the step.  A larger e, or
+// a u that does not have unit length to start with, is renormalised after
+// each substep.
+//
+// The coefficients belong to the length, so a step of n equal substeps forms
+// them once; a substep is then 14 FP64 operations along a coordinate axis
+// and 33 for any field direction, three deep, against 72 with a square root
+// and three divisions stage by stage.  Error against 128-bit arithmetic,
+// 4,000 tracks of 1-100 substeps: position 1.8e-14 cm rms, direction 1.0e-16;
+// stage by stage 1.8e-14 and 2.2e-16.  Calorimeter in 2 T, 4,000 events: 384 ms
+// stage by stage, 163 with the map and an explicit renormalisation per
+// substep, 142 like this (with the 32-bit chord test).
 struct FieldMap {
-    double h;         // displacement along u
-    double hp;        // h (1 - t^2/6): along u, components across the field
-    double x1, x2;    // displacement along w1, w2
-    double u1, u2;    // turn along w1, w2
+    double h;        // displacement along u
+    double hp;       // h (1 - t^2/6): along u, components across the field
+    double x1, x2;   // displacement along w1, w2
+    double c;        // u' / |u'| = u' + c u'
+    double u1, u2;   // turn along w1, w2 (with the factor 1 + c)
+    double ua, sa;   // axis field: u along the axis at the start, its growth per path
+    bool renormalise;  // after every substep
 };
 
-__device__ __forceinline__ FieldMap field_step(const Params<double>& p, double kq, double h, double)
+__device__ __forceinline__ FieldMap field_step(const Params<double>& p, double kq, double h, const double* u)
 {
     FieldMap f;
-    const double t = kq * (p.baxis >= 0 ? p.B[p.baxis] : p.bmag) * h;
+    const double k = kq * (p.baxis >= 0 ? p.B[p.baxis] : p.bmag);
+    const double t = k * h;
     const double tt = t * t;
     f.h = h;
     f.x2 = h * (tt * (1.0 / 6.0));
@@ -936,60 +964,83 @@ __device__ __forceinline__ FieldMap field_step(const Params<double>& p, double k
     f.x1 = h * (t * fma(tt, -1.0 / 24.0, 0.5));
     f.u1 = t * fma(tt, -1.0 / 6.0, 1.0);
     f.u2 = tt * fma(tt, -1.0 / 24.0, 0.5);
+    // e = g t^2 with |w1|^2 = |u|^2 - (u b)^2
+    const double uu = fma(u[0], u[0], fma(u[1], u[1], u[2] * u[2]));
+    const double ub = p.baxis < 0 ? fma(u[0], p.bhat[0], fma(u[1], p.bhat[1], u[2] * p.bhat[2]))
+                                  : (p.baxis == 0 ? u[0] : (p.baxis == 1 ? u[1] : u[2]));
+    const double g = tt * tt * fma(tt, 1.0 / 576.0, -1.0 / 72.0) * fma(-ub, ub, uu);
+    f.renormalise = !(fabs(g * tt) < 0x1p-27 && fabs(uu - 1.0) < 0x1p-48);
+    f.c = f.renormalise ? 0.0 : -0.5 * g * tt;
+    f.ua = ub;
+    f.sa = f.renormalise ? 0.0 : -0.5 * g * t * k * ub;
+    f.u1 = fma(f.c, f.u1, f.u1);
+    f.u2 = fma(-f.c, 1.0 - f.u2, f.u2);  // along -w2: u' + c u' = u - (u2 - c (1 - u2)) u + ...
     return f;
 }
 
 // field along axis A (its sign is in the coefficients): w1 = (0, u_k, -u_j),
 // w2 = -(0, u_j, u_k) in the cyclic order A, j, k
 template <int A>
-__device__ __forceinline__ void field_map_axis(const FieldMap& f, const double x[3], const double u[3], double xo[3],
-                                               double uo[3])
+__device__ __forceinline__ void field_map_axis(const FieldMap& f, double s, const double x[3], const double u[3],
+                                               double xo[3], double uo[3])
 {
     constexpr int J = (A + 1) % 3, K = (A + 2) % 3;
     xo[A] = fma(f.h, u[A], x[A]);
     xo[J] = x[J] + fma(f.x1, u[K], f.hp * u[J]);
     xo[K] = x[K] + fma(-f.x1, u[J], f.hp * u[K]);
-    uo[A] = u[A];
+    uo[A] = f.renormalise ? u[A] : fma(s, f.sa, f.ua);
     uo[J] = u[J] + fma(-f.u2, u[J], f.u1 * u[K]);
     uo[K] = u[K] - fma(f.u2, u[K], f.u1 * u[J]);
 }
 
-__device__ __forceinline__ void rk4(const Params<double>& p, const FieldMap& f, const double x[3], const double u[3],
-                                    double xo[3], double uo[3])
+// u / |u|: for a length within 2^-28 of 1 one fused multiply-add per
+// component, (1 + e)^(-1/2) being 1 - e/2 to within 2^-54.4
+__device__ __forceinline__ void renormalise(double u[3])
+{
+    const double n2 = fma(u[0], u[0], fma(u[1], u[1], u[2] * u[2]));
+    const double e = n2 - 1.0;
+    if ((__double2hiint(e) & 0x7FFFFFFF) < ((1023 - 27) << 20)) {
+        const double c = -0.5 * e;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) u[i] = fma(u[i], c, u[i]);
+    } else {
+        const auto nd = mdivisor(msqrt(n2));
+#pragma unroll
+        for (int i = 0; i < 3; ++i) u[i] = mdiv(u[i], nd);
+    }
+}
+
+// s: the path from the start of the step (of the map's u) to this substep's end
+__device__ __forceinline__ void rk4(const Params<double>& p, const FieldMap& f, double s, const double x[3],
+                                    const double u[3], double xo[3], double uo[3])
 {
     switch (p.baxis) {
-    case 0: field_map_axis<0>(f, x, u, xo, uo); break;
-    case 1: field_map_axis<1>(f, x, u, xo, uo); break;
-    case 2: field_map_axis<2>(f, x, u, xo, uo); break;
+    case 0: field_map_axis<0>(f, s, x, u, xo, uo); break;
+    case 1: field_map_axis<1>(f, s, x, u, xo, uo); break;
+    case 2: field_map_axis<2>(f, s, x, u, xo, uo); break;
     default: {
+        // w2 = (u b) b - u splits u' into parts along u, w1 and b w; formed
+        // as two cross products, which keep their size small against u
         const double* b = p.bhat;
         double w[3], v[3];
 #pragma unroll
         for (int i = 0; i < 3; ++i) w[i] = fma(u[(i + 1) % 3], b[(i + 2) % 3], -(u[(i + 2) % 3] * b[(i + 1) % 3]));
 #pragma unroll
         for (int i = 0; i < 3; ++i) v[i] = fma(w[(i + 1) % 3], b[(i + 2) % 3], -(w[(i + 2) % 3] * b[(i + 1) % 3]));
+        // along w2 the factor is u2 (1 + c): u2 here is u2 - c (1 - u2), so u2 + c
+        const double u2 = f.u2 + f.c;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             xo[i] = x[i] + fma(f.x2, v[i], fma(f.x1, w[i], f.h * u[i]));
-            uo[i] = u[i] + fma(f.u2, v[i], f.u1 * w[i]);
+            uo[i] = u[i] + fma(u2, v[i], fma(f.u1, w[i], f.c * u[i]));
         }
     }
     }
-    // Renormalise.  |u'|^2 = 1 + e with e of the order of t^6/72: below 2^-27
-    // the factor (1 + e)^(-1/2) is 1 - e/2 to within 2^-54.4, one fused
-    // multiply-add per component instead of a square root and divisions.
-    const double n2 = fma(uo[0], uo[0], fma(uo[1], uo[1], uo[2] * uo[2]));
-    const double e = n2 - 1.0;
-    if ((__double2hiint(e) & 0x7FFFFFFF) < ((1023 - 27) << 20)) {
-        const double c = -0.5 * e;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) uo[i] = fma(uo[i], c, uo[i]);
-    } else {
-        const auto nd = mdivisor(msqrt(n2));
-#pragma unroll
-        for (int i = 0; i < 3; ++i) uo[i] = mdiv(uo[i], nd);
-    }
+    if (f.renormalise) renormalise(uo);
 }
+
+// the end of a step: take off what rounding added to the length
+__device__ __forceinline__ void field_end(const FieldMap&, double u[3]) { renormalise(u); }
 
 // True when the chord from x (inside volume vol) to x1 cannot leave vol:
 // x1 lies inside the volume by more than kChordMargin, and in the world
@@ -1007,11 +1058,13 @@ constexpr double kChordMargin = 1e-6;  // cm
 // interaction: it bounds the work of one step of a looping track.
 constexpr int kMaxSubsteps = 100;
 
-// x1 lies more than kChordMargin inside a layer's side walls
+// True only when x1 lies more than kChordMargin inside a layer's side walls
+// (keys of 32 bits: false as well within their resolution of a wall, 1e-6 of
+// its distance; a false answer costs the full navigation and changes nothing)
 template <typename R>
 __device__ __forceinline__ bool inside_walls(const Params<R>& p, const double x1[3])
 {
-    const long long k0 = ord_key(x1[0]), k1 = ord_key(x1[1]);
+    const int k0 = ord_key(x1[0]), k1 = ord_key(x1[1]);
     return k0 > p.kxy[0] && k0 < p.kxy[1] && k1 > p.kxy[2] && k1 < p.kxy[3];
 }
 
@@ -1042,20 +1095,21 @@ __device__ __forceinline__ bool chord_inside(const Params<R>& p, int vol, const 
         }
         return true;
     }
-    // Layers: integer comparisons through ord_key, whose order is the numeric
-    // order of non-NaN values, with the bounds' keys formed when the geometry
-    // is loaded.  A NaN coordinate of x1 fails one of the tests of its axis.
+    // Layers: 32-bit integer comparisons through ord_key with the bounds' keys
+    // formed when the geometry is loaded (true only when the exact comparisons
+    // are).  A NaN coordinate of x1 fails one of the tests of its axis.
     if (vol >= 0) {
-        const long long k2 = ord_key(x1[2]);
-        return k2 > p.kz[2 * vol] && k2 < p.kz[2 * vol + 3] && inside_walls(p, x1);
+        const int k2 = ord_key(x1[2]);
+        const int2 z = p.kz[vol];
+        return k2 > z.x && k2 < z.y && inside_walls(p, x1);
     }
     bool inside = true, apart = false;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const long long k0 = ord_key(x[a]), k1 = ord_key(x1[a]);
+        const int k0 = ord_key(x[a]), k1 = ord_key(x1[a]);
         inside = inside && k1 > p.kworld[a][0] && k1 < p.kworld[a][1];
         // the chord and the layer stack are separated along axis a
-        apart = apart || (k0 < k1 ? k1 : k0) < p.kstack[a][0] || (k0 < k1 ? k0 : k1) > p.kstack[a][1];
+        apart = apart || max(k0, k1) < p.kstack[a][0] || min(k0, k1) > p.kstack[a][1];
     }
     return inside && apart;
 }
@@ -1071,31 +1125,25 @@ __device__ __forceinline__ double propagate_field(const Params<R>& p, int charge
     const double kq = mdiv(charge * kFieldC, pm);
     double s = 0.0;
     *crossed = false;
-    const auto whole = field_step(p, kq, hs, R(0));
+    const auto whole = field_step(p, kq, hs, u);
     for (int i = 0; i < n; ++i) {
         double x1[3];
         R u1[3];
-        rk4(p, whole, x, u, x1, u1);
+        rk4(p, whole, s + hs, x, u, x1, u1);
         *evals += 1;
+        double h = hs;
         if (!chord_inside<G>(p, vol, x, x1)) {
             double c[3];
 #pragma unroll
             for (int a = 0; a < 3; ++a) c[a] = x1[a] - x[a];
             const Exit e = nav_exit<G>(p, vol, x, c);
             if (e.t <= 1.0) {
-                const double h2 = hs * e.t;
-                rk4(p, field_step(p, kq, h2, R(0)), x, u, x1, u1);
+                h = hs * e.t;
+                rk4(p, field_step(p, kq, h, u), h, x, u, x1, u1);
                 *evals += 1;
                 snap(e, x1);
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    x[a] = x1[a];
-                    u[a] = u1[a];
-                }
-                s += h2;
                 *bnd = e;
                 *crossed = true;
-                return s;
             }
         }
 #pragma unroll
@@ -1103,8 +1151,10 @@ __device__ __forceinline__ double propagate_field(const Params<R>& p, int charge
             x[a] = x1[a];
             u[a] = u1[a];
         }
-        s += hs;
+        s += h;
+        if (*crossed) break;
     }
+    field_end(whole, u);
     return s;
 }
 
