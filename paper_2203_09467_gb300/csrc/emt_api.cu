@@ -43,9 +43,10 @@ struct Plan {
     size_t trk[2][11];
     size_t cnt, status, total_steps, done_head, ehist, gsync;
     size_t hist, ledger, counts, live, event_id, done_ring;
-    size_t grid, gridf, igrid, igridf, irs, irsf, tab, tabf, dedx, mats, bk, vacuum, x0, ray_a, scratch;
+    size_t grid, gridf, igrid, igridf, irs, irsf, tab, tabf, dedx, mats, bk, x0, ray_a, scratch;
     size_t dgrid, dgridf, dtab, dtabf;
-    size_t zb, kz, lmat, lbin;
+    size_t gnode, xnode, rnode, gnodef, xnodef, rnodef;
+    size_t zb, layer;
     size_t st_ev, st_type, st_T, st_pos, st_dir, st_uid, st_slot, st_ids, st_start, st_runs;
     size_t slots_tmp, out_hist, out_summary;
     size_t iq[13];      // split schedule: interaction queue fields
@@ -101,17 +102,20 @@ Plan make_plan(const emt_options& o)
     p.dgridf = p.add(kMaxGrid * sizeof(float));
     p.dtab = p.add((size_t)kMaxMat * 3 * kMaxGrid * kNq * sizeof(double));
     p.dtabf = p.add((size_t)kMaxMat * 3 * kMaxGrid * kNq * sizeof(float));
+    p.gnode = p.add(kMaxGrid * sizeof(Quad<double>));
+    p.xnode = p.add((size_t)kMaxMat * 3 * kMaxGrid * 2 * sizeof(Quad<double>));
+    p.rnode = p.add((size_t)kMaxMat * 3 * kMaxGrid * sizeof(Quad<double>));
+    p.gnodef = p.add(kMaxGrid * sizeof(Quad<float>));
+    p.xnodef = p.add((size_t)kMaxMat * 3 * kMaxGrid * 2 * sizeof(Quad<float>));
+    p.rnodef = p.add((size_t)kMaxMat * 3 * kMaxGrid * sizeof(Quad<float>));
     p.dedx = p.add((size_t)kMaxMat * 3 * kMaxGrid * sizeof(double));
     p.mats = p.add(kMaxMat * sizeof(MaterialDev));
     p.bk = p.add(kMaxMat * sizeof(double));
-    p.vacuum = p.add(kMaxMat * sizeof(int));
     p.x0 = p.add(kMaxMat * sizeof(double));
     p.ray_a = p.add(kMaxMat * sizeof(double));
     p.scratch = p.add((32 + (size_t)kMaxMat * 2 * kMaxGrid) * sizeof(double));
     p.zb = p.add((kMaxLayers + 1) * sizeof(double));
-    p.kz = p.add(kMaxLayers * sizeof(int2));
-    p.lmat = p.add(kMaxLayers * sizeof(int));
-    p.lbin = p.add(kMaxLayers * sizeof(int));
+    p.layer = p.add(kMaxLayers * sizeof(LayerRec));
     const size_t P = (size_t)p.max_prim;
     p.st_ev = p.add(P * 4);
     p.st_type = p.add(P * 4);
@@ -179,10 +183,10 @@ bool valid_options(const emt_options& o, std::string& why)
 }
 
 // Validate a geometry description and lay out its arrays: zb[n + 1] (plane
-// positions or shell radii), lm[n] (materials), lb[n] (score bins), and the
-// chord test's keys kz[n] of the planes.  Returns an error message, or nullptr.
+// positions or shell radii) and the layer records (materials as given, see
+// mark_vacuum).  Returns an error message, or nullptr.
 const char* check_geometry(const emt_layer* layers, int n, const emt_world* w, int n_mat, int max_bins, double* zb,
-                           int* lm, int* lb, int2* kz)
+                           LayerRec* rec)
 {
     if (n < 1 || n > kMaxLayers) return "layer count out of [1, 4096]";
     if (w->n_bins < 1 || w->n_bins > max_bins) return "n_bins out of [1, max_bins]";
@@ -195,10 +199,11 @@ const char* check_geometry(const emt_layer* layers, int n, const emt_world* w, i
         if (!(layers[i].thickness_cm > 0.0)) return "layer thickness must be positive";
         if (layers[i].material < -1 || layers[i].material >= n_mat) return "layer material index";
         zb[i + 1] = zb[i] + layers[i].thickness_cm;
-        lm[i] = layers[i].material;
-        lb[i] = layers[i].score_bin;
+        rec[i] = LayerRec{{zb[i], zb[i + 1]},
+                          layers[i].material,
+                          layers[i].score_bin,
+                          {ord_key(zb[i] + kChordMargin), ord_key(zb[i + 1] - kChordMargin)}};
     }
-    for (int i = 0; i < n; ++i) kz[i] = make_int2(ord_key(zb[i] + kChordMargin), ord_key(zb[i + 1] - kChordMargin));
     if (w->geometry == EMT_GEOM_LAYERS) {
         if (!(w->half_x_cm > 0.0) || !(w->half_y_cm > 0.0)) return "stack half widths";
         const double lo[3] = {-w->half_x_cm, -w->half_y_cm, zb[0]};
@@ -213,6 +218,13 @@ const char* check_geometry(const emt_layer* layers, int n, const emt_world* w, i
     if (b2 > 0.0 && (!(w->rk_delta_cm > 0.0) || !(w->max_field_step_cm > 0.0)))
         return "field needs rk_delta_cm > 0 and max_field_step_cm > 0";
     return nullptr;
+}
+
+// the step kernels' material index of a layer: -1 for a vacuum material
+void mark_vacuum(LayerRec* rec, int n, const int* vacuum)
+{
+    for (int i = 0; i < n; ++i)
+        if (rec[i].mat >= 0 && vacuum[rec[i].mat]) rec[i].mat = -1;
 }
 
 // Ends of the energy grid and find_bin's guess: with the FP32 bits i of E,
@@ -280,6 +292,8 @@ struct emt_ctx {
     bool poisoned = false;
     bool have_materials = false, have_geometry = false;
     int n_mat = 0, n_grid = 0, n_layers = 0, n_bins = 0;
+    int vacuum[kMaxMat] = {};       // material has no density
+    std::vector<LayerRec> layers;  // as loaded (a later load of materials marks vacuum anew)
     Params<double> pd;
     Params<float> pf;
     int64_t it = 0;  // step-loop iterations so far
@@ -426,13 +440,10 @@ void fill_common(emt_ctx* c, Params<R>& p)
     p.max_events = pl.max_events;
     p.seed = c->opt.seed;
     p.bk = c->at<double>(pl.bk);
-    p.vacuum = c->at<int>(pl.vacuum);
     p.x0 = c->at<double>(pl.x0);
     p.ray_a = c->at<double>(pl.ray_a);
     p.zb = c->at<double>(pl.zb);
-    p.kz = c->at<int2>(pl.kz);
-    p.lmat = c->at<int>(pl.lmat);
-    p.lbin = c->at<int>(pl.lbin);
+    p.layer = c->at<LayerRec>(pl.layer);
     p.step_bins = pl.step_bins;
     p.step_hist = pl.step_bins > 0 ? c->at<unsigned long long>(pl.step_hist) : nullptr;
     p.max_active = c->opt.max_active;
@@ -1121,7 +1132,8 @@ emt_status emt_load_materials(emt_ctx* c, const emt_material* mats, int32_t n, c
     if (!(ph->step_frac > 0.0) || !(ph->final_range_cm > 0.0)) return fail(c, EMT_ERR_INVALID_ARG, "step limits");
     std::vector<MaterialDev> md(n);
     std::vector<double> bk(n);
-    std::vector<int> vac(n);
+    int vac[kMaxMat];
+    std::memcpy(vac, c->vacuum, sizeof vac);
     for (int i = 0; i < n; ++i) {
         const emt_material& m = mats[i];
         bool vacuum = !(m.rho_g_cm3 > 0.0);
@@ -1135,7 +1147,11 @@ emt_status emt_load_materials(emt_ctx* c, const emt_material* mats, int32_t n, c
     const Plan& pl = c->plan;
     EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.mats, md.data(), sizeof(MaterialDev) * n, cudaMemcpyHostToDevice, c->stream));
     EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.bk, bk.data(), sizeof(double) * n, cudaMemcpyHostToDevice, c->stream));
-    EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.vacuum, vac.data(), sizeof(int) * n, cudaMemcpyHostToDevice, c->stream));
+    std::vector<LayerRec> rec = c->layers;
+    mark_vacuum(rec.data(), (int)rec.size(), vac);
+    if (!rec.empty())
+        EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.layer, rec.data(), sizeof(LayerRec) * rec.size(),
+                                    cudaMemcpyHostToDevice, c->stream));
     TableBuild b;
     b.mats = c->at<MaterialDev>(pl.mats);
     b.n_mat = n;
@@ -1159,6 +1175,12 @@ emt_status emt_load_materials(emt_ctx* c, const emt_material* mats, int32_t n, c
     b.dtab = c->at<double>(pl.dtab);
     b.dgridf = c->mixed() ? c->at<float>(pl.dgridf) : nullptr;
     b.dtabf = c->mixed() ? c->at<float>(pl.dtabf) : nullptr;
+    b.gnode = c->at<Quad<double>>(pl.gnode);
+    b.xnode = c->at<Quad<double>>(pl.xnode);
+    b.rnode = c->at<Quad<double>>(pl.rnode);
+    b.gnodef = c->mixed() ? c->at<Quad<float>>(pl.gnodef) : nullptr;
+    b.xnodef = c->mixed() ? c->at<Quad<float>>(pl.xnodef) : nullptr;
+    b.rnodef = c->mixed() ? c->at<Quad<float>>(pl.rnodef) : nullptr;
     EMT_CUDA(c, build_tables(b, c->at<double>(pl.scratch), c->stream));
     // the ends of the grid as the kernels see them (kernel parameters)
     double ends[2] = {0.0, 0.0};
@@ -1171,24 +1193,19 @@ emt_status emt_load_materials(emt_ctx* c, const emt_material* mats, int32_t n, c
     }
     EMT_CUDA(c, cudaStreamSynchronize(c->stream));
     c->n_mat = n;
+    std::memcpy(c->vacuum, vac, sizeof vac);
     c->n_grid = n_grid;
     for (int k = 0; k < 3; ++k) {
         c->pd.cut[k] = ph->cut_MeV[k];
         c->pf.cut[k] = ph->cut_MeV[k];
         c->pd.cutf[k] = c->pf.cutf[k] = (float)ph->cut_MeV[k];
     }
-    c->pd.grid = b.grid;
-    c->pd.tab = b.tab;
-    c->pf.grid = c->at<float>(pl.gridf);
-    c->pf.tab = c->at<float>(pl.tabf);
-    c->pd.igrid = b.igrid;
-    c->pd.irs = b.irs;
-    c->pf.igrid = c->at<float>(pl.igridf);
-    c->pf.irs = c->at<float>(pl.irsf);
-    c->pd.dgrid = b.dgrid;
-    c->pd.dtab = b.dtab;
-    c->pf.dgrid = c->at<float>(pl.dgridf);
-    c->pf.dtab = c->at<float>(pl.dtabf);
+    c->pd.gnode = b.gnode;
+    c->pd.xnode = b.xnode;
+    c->pd.rnode = b.rnode;
+    c->pf.gnode = c->at<Quad<float>>(pl.gnodef);
+    c->pf.xnode = c->at<Quad<float>>(pl.xnodef);
+    c->pf.rnode = c->at<Quad<float>>(pl.rnodef);
     c->pd.n_grid = c->pf.n_grid = n_grid;
     set_bin_guess(c->pd, ends[0], ends[1], ph->bins_per_decade);
     set_bin_guess(c->pf, endsf[0], endsf[1], ph->bins_per_decade);
@@ -1209,18 +1226,17 @@ emt_status emt_load_geometry(emt_ctx* c, const emt_layer* layers, int32_t n, con
     if (!c->have_materials) return fail(c, EMT_ERR_BAD_STATE, "load materials first");
     if (n < 1 || n > kMaxLayers) return fail(c, EMT_ERR_INVALID_ARG, "layer count out of [1, 4096]");
     std::vector<double> zb(n + 1);
-    std::vector<int> lm(n), lb(n);
-    std::vector<int2> kz(n);
-    if (const char* why =
-            check_geometry(layers, n, w, c->n_mat, c->opt.max_bins, zb.data(), lm.data(), lb.data(), kz.data()))
+    std::vector<LayerRec> rec(n);
+    if (const char* why = check_geometry(layers, n, w, c->n_mat, c->opt.max_bins, zb.data(), rec.data()))
         return fail(c, EMT_ERR_INVALID_ARG, why);
     if (cudaSetDevice(c->opt.device) != cudaSuccess) return fail(c, EMT_ERR_CUDA, "cudaSetDevice");
     const Plan& pl = c->plan;
     EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.zb, zb.data(), sizeof(double) * (n + 1), cudaMemcpyHostToDevice, c->stream));
-    EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.lmat, lm.data(), sizeof(int) * n, cudaMemcpyHostToDevice, c->stream));
-    EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.lbin, lb.data(), sizeof(int) * n, cudaMemcpyHostToDevice, c->stream));
-    EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.kz, kz.data(), sizeof(int2) * kz.size(), cudaMemcpyHostToDevice, c->stream));
+    std::vector<LayerRec> marked = rec;
+    mark_vacuum(marked.data(), n, c->vacuum);
+    EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.layer, marked.data(), sizeof(LayerRec) * n, cudaMemcpyHostToDevice, c->stream));
     EMT_CUDA(c, cudaStreamSynchronize(c->stream));
+    c->layers = std::move(rec);
     set_geometry(c->pd, n, w, zb.data());
     set_geometry(c->pf, n, w, zb.data());
     c->n_layers = n;
@@ -1706,8 +1722,7 @@ extern "C" emt_status emt_transport_static(int32_t device, uint32_t seed, const 
         vac[i] = vacuum ? 1 : 0;
     }
     if (cudaMemcpyAsync(pool + pl.mats, md, sizeof(MaterialDev) * n_mat, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(pool + pl.bk, bk, sizeof(double) * n_mat, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(pool + pl.vacuum, vac, sizeof(int) * n_mat, cudaMemcpyHostToDevice, st) != cudaSuccess)
+        cudaMemcpyAsync(pool + pl.bk, bk, sizeof(double) * n_mat, cudaMemcpyHostToDevice, st) != cudaSuccess)
         return EMT_ERR_CUDA;
     TableBuild b;
     b.mats = reinterpret_cast<const MaterialDev*>(pool + pl.mats);
@@ -1732,6 +1747,10 @@ extern "C" emt_status emt_transport_static(int32_t device, uint32_t seed, const 
     b.dtab = reinterpret_cast<double*>(pool + pl.dtab);
     b.dgridf = nullptr;
     b.dtabf = nullptr;
+    b.gnode = reinterpret_cast<Quad<double>*>(pool + pl.gnode);
+    b.xnode = reinterpret_cast<Quad<double>*>(pool + pl.xnode);
+    b.rnode = reinterpret_cast<Quad<double>*>(pool + pl.rnode);
+    b.gnodef = b.xnodef = b.rnodef = nullptr;
     double ends[2] = {0.0, 0.0};
     if (build_tables(b, reinterpret_cast<double*>(pool + pl.scratch), st) != cudaSuccess ||
         cudaMemcpyAsync(&ends[0], b.grid, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -1743,12 +1762,9 @@ extern "C" emt_status emt_transport_static(int32_t device, uint32_t seed, const 
         p.cut[k] = ph->cut_MeV[k];
         p.cutf[k] = (float)ph->cut_MeV[k];
     }
-    p.grid = b.grid;
-    p.tab = b.tab;
-    p.igrid = b.igrid;
-    p.irs = b.irs;
-    p.dgrid = b.dgrid;
-    p.dtab = b.dtab;
+    p.gnode = b.gnode;
+    p.xnode = b.xnode;
+    p.rnode = b.rnode;
     p.n_grid = n_grid;
     p.step_frac = ph->step_frac;
     p.final_range = ph->final_range_cm;
@@ -1758,14 +1774,11 @@ extern "C" emt_status emt_transport_static(int32_t device, uint32_t seed, const 
 
     // ---- geometry
     double zb[kMaxLayers + 1];
-    int lm[kMaxLayers], lb[kMaxLayers];
-    int2 kz[kMaxLayers];
-    if (check_geometry(layers, n_layers, w, n_mat, EMT_STATIC_MAX_BINS, zb, lm, lb, kz)) return EMT_ERR_INVALID_ARG;
+    LayerRec rec[kMaxLayers];
+    if (check_geometry(layers, n_layers, w, n_mat, EMT_STATIC_MAX_BINS, zb, rec)) return EMT_ERR_INVALID_ARG;
+    mark_vacuum(rec, n_layers, vac);
     if (cudaMemcpyAsync(pool + pl.zb, zb, sizeof(double) * (n_layers + 1), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(pool + pl.kz, kz, sizeof(int2) * n_layers, cudaMemcpyHostToDevice, st) !=
-            cudaSuccess ||
-        cudaMemcpyAsync(pool + pl.lmat, lm, sizeof(int) * n_layers, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(pool + pl.lbin, lb, sizeof(int) * n_layers, cudaMemcpyHostToDevice, st) != cudaSuccess)
+        cudaMemcpyAsync(pool + pl.layer, rec, sizeof(LayerRec) * n_layers, cudaMemcpyHostToDevice, st) != cudaSuccess)
         return EMT_ERR_CUDA;
     set_geometry(p, n_layers, w, zb);
 

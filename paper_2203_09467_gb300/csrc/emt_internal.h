@@ -35,6 +35,8 @@ struct TableBuild {
     double* dtab;   // [n_mat][3][n_grid][4] tab[n+1][q] - tab[n][q] (last node 0)
     float* dgridf;  // optional: the same differences of the float copies, in float
     float* dtabf;
+    Quad<double>*gnode, *xnode, *rnode;  // lookup records of the step kernels (Params)
+    Quad<float>*gnodef, *xnodef, *rnodef;  // optional
 };
 
 // scratch: (32 + n_mat * 2 * n_grid) doubles

@@ -186,33 +186,34 @@ __device__ __forceinline__ int transport_part(const Params<R>& p, TrackReg<R>& t
     const uint64_t event_id = p.event_id[t.ev];
     Draws dr;
     dr.init(p.seed, event_id, t.uid, t.step);
-    const int mi = t.vol >= 0 ? p.lmat[t.vol] : -1;
-    const bool matter = mi >= 0 && !p.vacuum[mi];
+    LayerRec here;
+    here.mat = here.bin = -1;
+    if (t.vol >= 0) here = p.layer[t.vol];
+    const int mi = here.mat;
+    const bool matter = mi >= 0;
     const bool charged = t.type != 0;
     // photons: photo, Compton, pair (+ Rayleigh); e-: ioni, brems; e+: ioni,
     // brems, annihilation
     const int nproc = t.type == 1 ? 2 : ((X && t.type == 0 && (p.mask & kProcRayleigh)) ? 4 : 3);
-    const size_t row = matter ? (size_t)(mi * 3 + t.type) * p.n_grid * kNq : 0;
-    const R* tab = p.tab + row;
-    const R* dtab = p.dtab + row;
+    const int row = matter ? mi * 3 + t.type : 0;
 
     // cumulative cross sections in the order of the processes: cum[i] is the
     // sum of the first i + 1, the last of them the total
     R cum[4] = {R(0), R(0), R(0), R(0)};
     R sig_tot = R(0);
     R Rng = R(0);
-    Lookup<R> lk;
-    lk.n = 0;
-    lk.f = R(0);
-    lk.clamp = -1;
+    int interval = 0;
     if (matter) {
-        lk = locate_energy(p, t.T);
-        cum[0] = xs_value(p, tab, dtab, lk, 0);
-        cum[1] = sig_tot = cum[0] + xs_value(p, tab, dtab, lk, 1);
-        if (nproc >= 3) cum[2] = sig_tot = sig_tot + xs_value(p, tab, dtab, lk, 2);
+        const Lookup<R> lk = locate_energy(p, t.T);
+        const XsNode<R> xs = load_xs(p, row, lk.xn);
+        interval = lk.n;
+        cum[0] = xs_value(xs, lk.f, 0);
+        cum[1] = sig_tot = cum[0] + xs_value(xs, lk.f, 1);
+        if (nproc >= 3) cum[2] = sig_tot = sig_tot + xs_value(xs, lk.f, 2);
         if constexpr (X) {
-            if (nproc == 4) cum[3] = sig_tot = sig_tot + xs_value(p, tab, dtab, lk, 3);
+            if (nproc == 4) cum[3] = sig_tot = sig_tot + xs_value(xs, lk.f, 3);
         }
+        if (charged) Rng = range_value(p, xs, row, t.T, lk);
     }
     const R kInf = R(__longlong_as_double(0x7FF0000000000000ll));
     R s_int = kInf;
@@ -234,7 +235,6 @@ __device__ __forceinline__ int transport_part(const Params<R>& p, TrackReg<R>& t
     }
     R s_max = kInf;
     if (charged && matter) {
-        Rng = range_value(p, tab, dtab, t.T, lk);
         R fr_lim = pfinal_range(p);
         R lim = lt_pos(Rng, fr_lim) ? Rng : fr_lim;
         R fr = pstep_frac(p) * Rng;
@@ -288,7 +288,7 @@ __device__ __forceinline__ int transport_part(const Params<R>& p, TrackReg<R>& t
             bool done = false;
             if (t.vol >= 0 && nonzero(ud[2])) {
                 const bool up = gt_zero(ud[2]);
-                const double pl = p.zb[t.vol + (up ? 1 : 0)];
+                const double pl = up ? here.z[1] : here.z[0];
                 double te = mdiv(pl - t.x[2], ud[2]);
                 if (__double_as_longlong(te) < 0) te = 0.0;
                 boundary = le_pos(te, s_physd);
@@ -342,14 +342,14 @@ __device__ __forceinline__ int transport_part(const Params<R>& p, TrackReg<R>& t
         boundary = crossed;
     }
     if (boundary) interact = false;
-    fx.col = score_col(p, t.vol, t.x[2]);
+    fx.col = score_col_bin(p, here.bin, t.x[2]);
 
     alive = true;
     const R T0 = t.T;
     // 6-7: continuous loss
     if (charged && matter) {
         R r = Rng - from_d<R>(s);
-        R Tn = gt_zero(r) ? inv_range(p, tab, p.irs + (size_t)(mi * 3 + t.type) * p.n_grid, r, lk.n) : R(0);
+        R Tn = gt_zero(r) ? inv_range(p, row, r, interval) : R(0);
         R ed = t.T - Tn;
         fx.dep = to_d(ed);  // 0 + ed: ed is never -0
         t.T = Tn;
@@ -433,14 +433,14 @@ __device__ __forceinline__ void interaction_part(const Params<R>& p, TrackReg<R>
     const R T = t.T;
     const R cut_e = pcut(p, 1), kc = pcut(p, 0);
     switch (m) {
-    case kPhoto: sample_photo(dr, T, from_d<R>(p.bk[p.lmat[t.vol]]), t.u, pr, angular); break;
+    case kPhoto: sample_photo(dr, T, from_d<R>(p.bk[p.layer[t.vol].mat]), t.u, pr, angular); break;
     case kCompton: sample_compton(dr, T, t.u, pr, t.T); break;
     case kPair: sample_pair(dr, T, t.u, pr, angular); break;
     case kMoller: sample_moller(dr, T, cut_e, t.u, pr, t.T); break;
     case kBhabha: sample_bhabha(dr, T, cut_e, t.u, pr, t.T); break;
     case kBrems: sample_brems(dr, T, kc, t.u, pr, t.T, angular); break;
     case kRayleigh:
-        if constexpr (X) sample_rayleigh(dr, T, from_d<R>(p.ray_a[p.lmat[t.vol]]), t.u);
+        if constexpr (X) sample_rayleigh(dr, T, from_d<R>(p.ray_a[p.layer[t.vol].mat]), t.u);
         break;
     default: sample_annih(dr, T, t.u, pr); break;
     }
@@ -511,17 +511,18 @@ __device__ __forceinline__ int field_substeps_estimate(const Params<R>& p, const
     const float pm = sqrtf(T * (T + 2.0f * (float)kMe));
     const float hmax = sqrtf(8.0f * (pm / ((float)kFieldC * (float)p.bmag)) * (float)p.rk_delta);
     float s = fminf((float)p.max_field_step, (float)kMaxSubsteps * hmax);
-    const int mi = t.vol >= 0 ? p.lmat[t.vol] : -1;
-    if (mi >= 0 && !p.vacuum[mi]) {
-        const size_t row = (size_t)(mi * 3 + t.type) * p.n_grid * kNq;
-        const R* tab = p.tab + row;
-        const R* dtab = p.dtab + row;
+    LayerRec here;
+    here.mat = -1;
+    if (t.vol >= 0) here = p.layer[t.vol];
+    if (here.mat >= 0) {
+        const int row = here.mat * 3 + t.type;
         const Lookup<R> lk = locate_energy(p, t.T);
-        const float rng = est_f(range_value(p, tab, dtab, t.T, lk));
+        const XsNode<R> xs = load_xs(p, row, lk.xn);
+        const float rng = est_f(range_value(p, xs, row, t.T, lk));
         const float lim = fminf(rng, est_f(pfinal_range(p)));
         s = fminf(s, fmaxf(est_f(pstep_frac(p)) * rng, lim));
-        float sig = est_f(xs_value(p, tab, dtab, lk, 0)) + est_f(xs_value(p, tab, dtab, lk, 1));
-        if (t.type == 2) sig += est_f(xs_value(p, tab, dtab, lk, 2));
+        float sig = est_f(xs_value(xs, lk.f, 0)) + est_f(xs_value(xs, lk.f, 1));
+        if (t.type == 2) sig += est_f(xs_value(xs, lk.f, 2));
         if (sig > 0.0f) {
             Draws dr;
             dr.init(p.seed, p.event_id[t.ev], t.uid, t.step);
@@ -536,8 +537,8 @@ __device__ __forceinline__ int field_substeps_estimate(const Params<R>& p, const
         const float uz = est_f(t.u[2]);
         const float z = (float)t.x[2];
         float dz = 3.0e38f;
-        if (uz > 0.0f) dz = ((float)p.zb[t.vol + 1] - z) / uz;
-        if (uz < 0.0f) dz = (z - (float)p.zb[t.vol]) / -uz;
+        if (uz > 0.0f) dz = ((float)here.z[1] - z) / uz;
+        if (uz < 0.0f) dz = (z - (float)here.z[0]) / -uz;
         s = fminf(s, fmaxf(dz, 0.0f) + hmax);
     }
     const float n = ceilf(s / hmax);

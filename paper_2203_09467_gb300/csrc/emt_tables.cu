@@ -345,6 +345,22 @@ __global__ void k_node_diff(const T* v, T* d, int total, int n, int q)
     d[idx] = i + 1 < n ? v[idx + q] - v[idx] : T(0);
 }
 
+// the lookup records of the step kernels from the separate tables (emt_device.cuh, Params)
+template <typename R>
+__global__ void k_pack(int rows, int n, const R* grid, const R* igrid, const R* dgrid, const R* tab, const R* dtab,
+                       const R* irs, Quad<R>* gnode, Quad<R>* xnode, Quad<R>* rnode)
+{
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= rows * n) return;
+    const int i = idx % n;
+    if (idx < n) gnode[i] = Quad<R>{grid[i], igrid[i], dgrid[i], R(0)};
+    const R* v = tab + (size_t)idx * kNq;
+    const R* d = dtab + (size_t)idx * kNq;
+    xnode[2 * (size_t)idx + 0] = Quad<R>{v[0], d[0], v[1], d[1]};
+    xnode[2 * (size_t)idx + 1] = Quad<R>{v[2], d[2], v[3], d[3]};
+    rnode[idx] = Quad<R>{v[3], irs[idx], grid[i], dgrid[i]};
+}
+
 }  // namespace
 
 // reciprocal interval widths of the energy grid and of the range tables
@@ -393,6 +409,8 @@ cudaError_t build_tables(const TableBuild& b, double* scratch, cudaStream_t st)
     const int nt = b.n_mat * 3 * b.n_grid * kNq;
     k_node_diff<<<(nt + 255) / 256, 256, 0, st>>>(b.tab, b.dtab, nt, b.n_grid, kNq);
     k_node_diff<<<(b.n_grid + 255) / 256, 256, 0, st>>>(b.grid, b.dgrid, b.n_grid, b.n_grid, 1);
+    k_pack<<<(nr + 127) / 128, 128, 0, st>>>(b.n_mat * 3, b.n_grid, b.grid, b.igrid, b.dgrid, b.tab, b.dtab, b.irs,
+                                             b.gnode, b.xnode, b.rnode);
     if (b.tabf) {
         k_to_float<<<(nt + 255) / 256, 256, 0, st>>>(b.tab, b.tabf, nt);
         k_to_float<<<(b.n_grid + 255) / 256, 256, 0, st>>>(b.grid, b.gridf, b.n_grid);
@@ -400,6 +418,8 @@ cudaError_t build_tables(const TableBuild& b, double* scratch, cudaStream_t st)
         k_to_float<<<(nr + 255) / 256, 256, 0, st>>>(b.irs, b.irsf, nr);
         k_node_diff<<<(nt + 255) / 256, 256, 0, st>>>(b.tabf, b.dtabf, nt, b.n_grid, kNq);
         k_node_diff<<<(b.n_grid + 255) / 256, 256, 0, st>>>(b.gridf, b.dgridf, b.n_grid, b.n_grid, 1);
+        k_pack<<<(nr + 127) / 128, 128, 0, st>>>(b.n_mat * 3, b.n_grid, b.gridf, b.igridf, b.dgridf, b.tabf, b.dtabf,
+                                                 b.irsf, b.gnodef, b.xnodef, b.rnodef);
     }
     return cudaGetLastError();
 }
