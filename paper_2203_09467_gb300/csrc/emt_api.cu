@@ -265,6 +265,8 @@ void set_geometry(Params<R>& p, int n, const emt_world* w, const double* zb)
     }
     p.bmag = std::sqrt(w->B_tesla[0] * w->B_tesla[0] + w->B_tesla[1] * w->B_tesla[1] + w->B_tesla[2] * w->B_tesla[2]);
     p.rk_delta = w->rk_delta_cm;
+    p.rk_delta8 = 8.0 * w->rk_delta_cm;
+    p.cb = kFieldC * p.bmag;
     p.max_field_step = w->max_field_step_cm;
     p.has_field = p.bmag > 0.0 ? 1 : 0;
     p.baxis = -1;

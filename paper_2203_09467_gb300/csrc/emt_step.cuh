@@ -316,7 +316,7 @@ __device__ __forceinline__ int transport_part(const Params<R>& p, TrackReg<R>& t
         }
     } else if constexpr (F) {
         double smax = s_physd;
-        if (smax > p.max_field_step) {
+        if (lt_pos(p.max_field_step, smax)) {
             smax = p.max_field_step;
             interact = false;
         }
@@ -324,18 +324,16 @@ __device__ __forceinline__ int transport_part(const Params<R>& p, TrackReg<R>& t
         // most kMaxSubsteps of them
         const double Td = to_d(t.T);
         const double pm = msqrt(Td * (Td + 2.0 * kMe));
-        const double hmax = msqrt(8.0 * mdiv(pm, kFieldC * p.bmag) * p.rk_delta);
+        const double hmax = msqrt(mdiv(pm, p.cb) * p.rk_delta8);
         int nsub;
         double hs;
-        if (smax > kMaxSubsteps * hmax) {
+        if (lt_pos(kMaxSubsteps * hmax, smax)) {
             nsub = kMaxSubsteps;
             hs = hmax;
             interact = false;
         } else {
-            double ns = ceil(mdiv(smax, hmax));
-            if (ns < 1.0) ns = 1.0;
-            nsub = (int)ns;
-            hs = mdiv(smax, ns);
+            nsub = ceil_count(mdiv(smax, hmax));
+            hs = mdiv(smax, small_int(nsub));
         }
         bool crossed = false;
         s = propagate_field<G>(p, t.type == 1 ? -1 : 1, pm, t.vol, t.x, t.u, nsub, hs, &e, &crossed, &fx.substeps);
