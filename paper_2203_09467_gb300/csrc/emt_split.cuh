@@ -427,21 +427,21 @@ __device__ __forceinline__ void interact_chunks(const Params<R>& p, const Tracks
             long long r = 0;
             if (mine) {
                 r = r0 + perm[pos];
-                const uint32_t tv = iq.tv[r];
-                t.x[0] = iq.x[r];
-                t.x[1] = iq.y[r];
-                t.x[2] = iq.z[r];
-                t.u[0] = iq.ux[r];
-                t.u[1] = iq.uy[r];
-                t.u[2] = iq.uz[r];
-                t.T = iq.T[r];
-                t.uid = iq.uid[r];
-                t.ev = iq.ev[r];
-                t.step = iq.step[r];
+                const uint32_t tv = __ldcg(iq.tv + r);
+                t.x[0] = __ldcg(iq.x + r);
+                t.x[1] = __ldcg(iq.y + r);
+                t.x[2] = __ldcg(iq.z + r);
+                t.u[0] = __ldcg(iq.ux + r);
+                t.u[1] = __ldcg(iq.uy + r);
+                t.u[2] = __ldcg(iq.uz + r);
+                t.T = __ldcg(iq.T + r);
+                t.uid = __ldcg(iq.uid + r);
+                t.ev = __ldcg(iq.ev + r);
+                t.step = __ldcg(iq.step + r);
                 t.type = (int)(tv & 0xFFu);
                 t.vol = (int)((tv >> 8) & 0xFFFFu) - 2;
-                rsrc = iq.src[r];
-                fx.dep = iq.dep[r];
+                rsrc = __ldcg(iq.src + r);
+                fx.dep = __ldcg(iq.dep + r);
                 fx.esc = 0.0;
                 fx.kill = 0.0;
                 fx.col = score_col(p, t.vol, t.x[2]);

@@ -543,20 +543,22 @@ __device__ __forceinline__ int field_substeps_estimate(const Params<R>& p, const
     return n < 1.0f ? 1 : (n > (float)kMaxSubsteps ? kMaxSubsteps : (int)n);
 }
 
+// Track and queue records are read once, past the L1, which is left to the
+// tables (FP64 and mixed calorimeter of 10,000 events 0.4 and 0.3% faster).
 template <typename R>
 __device__ __forceinline__ void load_track(const Tracks<R>& q, long long i, TrackReg<R>& t)
 {
-    t.x[0] = q.x[i];
-    t.x[1] = q.y[i];
-    t.x[2] = q.z[i];
-    t.u[0] = q.ux[i];
-    t.u[1] = q.uy[i];
-    t.u[2] = q.uz[i];
-    t.T = q.T[i];
-    t.uid = q.uid[i];
-    t.ev = q.ev[i];
-    t.step = q.step[i];
-    uint32_t tv = q.tv[i];
+    t.x[0] = __ldcg(q.x + i);
+    t.x[1] = __ldcg(q.y + i);
+    t.x[2] = __ldcg(q.z + i);
+    t.u[0] = __ldcg(q.ux + i);
+    t.u[1] = __ldcg(q.uy + i);
+    t.u[2] = __ldcg(q.uz + i);
+    t.T = __ldcg(q.T + i);
+    t.uid = __ldcg(q.uid + i);
+    t.ev = __ldcg(q.ev + i);
+    t.step = __ldcg(q.step + i);
+    uint32_t tv = __ldcg(q.tv + i);
     t.type = tv_type(tv);
     t.vol = tv_vol(tv);
 }
