@@ -1061,21 +1061,24 @@ emt_status emt_create(const emt_options* o, emt_ctx** out)
     auto resident = [&](auto per_sm_f, auto per_sm_d) {
         return std::max(1, dev_sms * (c->mixed() ? per_sm_f() : per_sm_d()));
     };
+    const bool select = o->max_active > 0;
     for (int f = 0; f < 2; ++f) {
         const bool field = f != 0;
         const int bs = c->block;
-        c->resident_blocks[f] = resident([&] { return Launch<float>::max_blocks_per_sm(bs, field); },
-                                         [&] { return Launch<double>::max_blocks_per_sm(bs, field); });
-        if (c->plan.split)
-            c->resident_a[f] = resident([&] { return Launch<float>::max_blocks_split(bs, 0, field); },
-                                        [&] { return Launch<double>::max_blocks_split(bs, 0, field); });
-        if (c->plan.pipelined)
+        // only the kernels that this context can launch are asked for
+        if (!c->plan.split)
+            c->resident_blocks[f] = resident([&] { return Launch<float>::max_blocks_per_sm(bs, field); },
+                                             [&] { return Launch<double>::max_blocks_per_sm(bs, field); });
+        else if (!c->plan.pipelined)
+            c->resident_a[f] = resident([&] { return Launch<float>::max_blocks_transport(bs, field, select); },
+                                        [&] { return Launch<double>::max_blocks_transport(bs, field, select); });
+        else
             c->resident_p[f] = resident([&] { return Launch<float>::max_blocks_pipe(bs, field); },
                                         [&] { return Launch<double>::max_blocks_pipe(bs, field); });
     }
     if (c->plan.split)
-        c->resident_b = resident([&] { return Launch<float>::max_blocks_split(c->block, 1, false); },
-                                 [&] { return Launch<double>::max_blocks_split(c->block, 1, false); });
+        c->resident_b = resident([&] { return Launch<float>::max_blocks_interact(c->block, select); },
+                                 [&] { return Launch<double>::max_blocks_interact(c->block, select); });
     if (o->loop_mode == EMT_LOOP_PERSISTENT) {
         int coop = 0, clock_khz = 0;
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, o->device);
@@ -1184,15 +1187,12 @@ emt_status emt_load_materials(emt_ctx* c, const emt_material* mats, int32_t n, c
     b.xnodef = c->mixed() ? c->at<Quad<float>>(pl.xnodef) : nullptr;
     b.rnodef = c->mixed() ? c->at<Quad<float>>(pl.rnodef) : nullptr;
     EMT_CUDA(c, build_tables(b, c->at<double>(pl.scratch), c->stream));
-    // the ends of the grid as the kernels see them (kernel parameters)
-    double ends[2] = {0.0, 0.0};
-    float endsf[2] = {0.f, 0.f};
-    for (int k = 0; k < 2; ++k) {
-        const size_t node = k ? (size_t)n_grid - 1 : 0;
-        EMT_CUDA(c, cudaMemcpyAsync(&ends[k], b.grid + node, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-        if (c->mixed())
-            EMT_CUDA(c, cudaMemcpyAsync(&endsf[k], b.gridf + node, sizeof(float), cudaMemcpyDeviceToHost, c->stream));
-    }
+    // the ends of the grid as the kernels see them (kernel parameters):
+    // together in the first grid record
+    Quad<double> ends{};
+    Quad<float> endsf{};
+    EMT_CUDA(c, c->mixed() ? cudaMemcpyAsync(&endsf, b.gnodef, sizeof endsf, cudaMemcpyDeviceToHost, c->stream)
+                           : cudaMemcpyAsync(&ends, b.gnode, sizeof ends, cudaMemcpyDeviceToHost, c->stream));
     EMT_CUDA(c, cudaStreamSynchronize(c->stream));
     c->n_mat = n;
     std::memcpy(c->vacuum, vac, sizeof vac);
@@ -1209,8 +1209,10 @@ emt_status emt_load_materials(emt_ctx* c, const emt_material* mats, int32_t n, c
     c->pf.xnode = c->at<Quad<float>>(pl.xnodef);
     c->pf.rnode = c->at<Quad<float>>(pl.rnodef);
     c->pd.n_grid = c->pf.n_grid = n_grid;
-    set_bin_guess(c->pd, ends[0], ends[1], ph->bins_per_decade);
-    set_bin_guess(c->pf, endsf[0], endsf[1], ph->bins_per_decade);
+    if (c->mixed())
+        set_bin_guess(c->pf, endsf.a, endsf.d, ph->bins_per_decade);
+    else
+        set_bin_guess(c->pd, ends.a, ends.d, ph->bins_per_decade);
     c->pd.step_frac = c->pf.step_frac = ph->step_frac;
     c->pd.mask = c->pf.mask = ph->process_mask;
     c->pd.final_range = c->pf.final_range = ph->final_range_cm;
@@ -1753,13 +1755,12 @@ extern "C" emt_status emt_transport_static(int32_t device, uint32_t seed, const 
     b.xnode = reinterpret_cast<Quad<double>*>(pool + pl.xnode);
     b.rnode = reinterpret_cast<Quad<double>*>(pool + pl.rnode);
     b.gnodef = b.xnodef = b.rnodef = nullptr;
-    double ends[2] = {0.0, 0.0};
+    Quad<double> ends{};
     if (build_tables(b, reinterpret_cast<double*>(pool + pl.scratch), st) != cudaSuccess ||
-        cudaMemcpyAsync(&ends[0], b.grid, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(&ends[1], b.grid + n_grid - 1, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaMemcpyAsync(&ends, b.gnode, sizeof ends, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
         return EMT_ERR_CUDA;
-    set_bin_guess(p, ends[0], ends[1], ph->bins_per_decade);
+    set_bin_guess(p, ends.a, ends.d, ph->bins_per_decade);
     for (int k = 0; k < 3; ++k) {
         p.cut[k] = ph->cut_MeV[k];
         p.cutf[k] = (float)ph->cut_MeV[k];

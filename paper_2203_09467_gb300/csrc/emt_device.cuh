@@ -256,7 +256,7 @@ template <typename R>
 struct Params {
     // tables, n_grid nodes each; d* is the difference to the next node (0 at
     // the last), formed once with the lookup's own subtraction
-    const Quad<R>* gnode;  // {E, 1/dE, dE, 0} of the energy grid
+    const Quad<R>* gnode;  // {E, 1/dE, dE, last E} of the energy grid
     const Quad<R>* xnode;  // [m * 3 + p][node][2]: {v0, dv0, v1, dv1}, {v2, dv2, v3, dv3}
     const Quad<R>* rnode;  // [m * 3 + p][node]: {R, 1/dR, E, dE} of the range tables
     int n_grid;

@@ -58,7 +58,8 @@ struct Launch {
     // split schedule: transport kernel then interaction kernel
     static cudaError_t step_split(const Params<R>& p, int side, int cin, int cout, int cclr, int grid_a, int grid_b,
                                   int block, cudaStream_t st);
-    static int max_blocks_split(int block, int which, bool field);
+    static int max_blocks_transport(int block, bool field, bool select);
+    static int max_blocks_interact(int block, bool select);
     // pipelined schedule: one kernel per step (plus the two sorting launches
     // of the charged tracks in a field, on grid_sort blocks)
     static cudaError_t step_pipe(const Params<R>& p, int side, int cin, int cout, int cclr, int grid, int grid_sort,

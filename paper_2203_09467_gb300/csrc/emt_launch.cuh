@@ -187,28 +187,32 @@ cudaError_t Launch<R>::step_split(const Params<R>& p, int side, int cin, int cou
                             : launch_split<R, false>(p, side, cin, cout, cclr, grid_a, grid_b, block, st);
 }
 
-// resident blocks per SM of the split kernels (which 0: transport, 1:
-// interaction)
+// resident blocks per SM of the split kernels, with or without track selection
 template <typename R>
-int Launch<R>::max_blocks_split(int block, int which, bool field)
+int Launch<R>::max_blocks_transport(int block, bool field, bool select)
 {
     int n = 0;
     with_block(block, [&](auto bs) {
         constexpr int kBs = decltype(bs)::value;
-        if (which == 0) {
-            const int all = min_blocks(kBs, field, [](auto g, auto f, auto x) {
-                return k_transport<R, kBs, g.value, f.value, false, x.value>;
-            });
-            const int selected = min_blocks(kBs, field, [](auto g, auto f, auto x) {
-                return k_transport<R, kBs, g.value, f.value, true, x.value>;
-            });
-            n = all < selected ? all : selected;
-        } else {
-            const int all = min_blocks(kBs, field, [](auto, auto, auto x) { return k_interact<R, kBs, false, x.value>; });
-            const int selected =
-                min_blocks(kBs, field, [](auto, auto, auto x) { return k_interact<R, kBs, true, x.value>; });
-            n = all < selected ? all : selected;
-        }
+        n = select ? min_blocks(kBs, field, [](auto g, auto f, auto x) {
+                         return k_transport<R, kBs, g.value, f.value, true, x.value>;
+                     })
+                   : min_blocks(kBs, field, [](auto g, auto f, auto x) {
+                         return k_transport<R, kBs, g.value, f.value, false, x.value>;
+                     });
+        return cudaSuccess;
+    });
+    return n > 0 ? n : 1;
+}
+
+template <typename R>
+int Launch<R>::max_blocks_interact(int block, bool select)
+{
+    int n = 0;
+    with_block(block, [&](auto bs) {
+        constexpr int kBs = decltype(bs)::value;
+        n = select ? min_blocks(kBs, false, [](auto, auto, auto x) { return k_interact<R, kBs, true, x.value>; })
+                   : min_blocks(kBs, false, [](auto, auto, auto x) { return k_interact<R, kBs, false, x.value>; });
         return cudaSuccess;
     });
     return n > 0 ? n : 1;
@@ -260,7 +264,8 @@ int Launch<R>::max_blocks_pipe(int block, bool field)
     template int Launch<R>::persist_blocks_per_sm(int, bool);
 #define EMT_INSTANTIATE_SPLIT(R)                                                                                    \
     template cudaError_t Launch<R>::step_split(const Params<R>&, int, int, int, int, int, int, int, cudaStream_t); \
-    template int Launch<R>::max_blocks_split(int, int, bool);
+    template int Launch<R>::max_blocks_transport(int, bool, bool);                                                 \
+    template int Launch<R>::max_blocks_interact(int, bool);
 #define EMT_INSTANTIATE_PIPE(R)                                                                                     \
     template cudaError_t Launch<R>::step_pipe(const Params<R>&, int, int, int, int, int, int, int, cudaStream_t);  \
     template int Launch<R>::max_blocks_pipe(int, bool);

@@ -353,7 +353,7 @@ __global__ void k_pack(int rows, int n, const R* grid, const R* igrid, const R* 
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= rows * n) return;
     const int i = idx % n;
-    if (idx < n) gnode[i] = Quad<R>{grid[i], igrid[i], dgrid[i], R(0)};
+    if (idx < n) gnode[i] = Quad<R>{grid[i], igrid[i], dgrid[i], grid[n - 1]};
     const R* v = tab + (size_t)idx * kNq;
     const R* d = dtab + (size_t)idx * kNq;
     xnode[2 * (size_t)idx + 0] = Quad<R>{v[0], d[0], v[1], d[1]};
