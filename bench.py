@@ -49,9 +49,10 @@ METRIC = "track-steps/s"
 # precision and step schedule.  Reported only while the kernel sources are
 # the ones that were measured (SHA-256 below).
 TRAFFIC = {
-    "kernel_sha256": "15abf5842738ce5d4e9c433fb3bef2edc32a6368716462450f708d34bdded67d",
-    "bytes_per_track_step": {"calo/fp64/pipelined": 101.6, "calo/fp64/split": 114.4, "calo/mixed/pipelined": 97.5,
-                             "calo_field/fp64/split": 109.1},
+    "kernel_sha256": "593ae42d8a938c3cf8c71ed485a153ae10b347872d2f8252545de94fcf743838",
+    "bytes_per_track_step": {"calo/fp64/pipelined": 129.2, "calo/fp64/split": 122.4, "calo/mixed/pipelined": 76.7,
+                             "calo/mixed/split": 86.6, "calo_field/fp64/split": 119.9,
+                             "calo_field/mixed/split": 82.4},
     "source": "profiles/step_kernels_dram_traffic.md",
 }
 # Algorithmic FP64 work of one track-step of the method, fixed by its
@@ -59,8 +60,12 @@ TRAFFIC = {
 # workload (oracle/census.py; summary in profiles/fp64_census_of_the_step.md),
 # in flops with add, sub, mul, div and sqrt one each and an fma two
 # (comparisons and elementary functions are listed there, not counted).  It
-# does not change when the kernels are optimised.
-FLOPS_PER_TRACK_STEP = {"calo": 43.09, "calo_field": 967.93, "cms": 73.49, "slab": 59.05, "batched": 969.84}
+# does not change when the kernels are optimised, except that the field
+# workloads count what a step needs once the RK4 stages of a uniform field are
+# collapsed to a linear map (emt_device.cuh): 23 flops per substep along an
+# axis, 7.16 substeps per track-step, 35 flops for the map, and the 43.1 of a
+# step without a field (stage by stage the census counts 968).
+FLOPS_PER_TRACK_STEP = {"calo": 43.09, "calo_field": 243.0, "cms": 73.49, "slab": 59.05, "batched": 243.0}
 # nominal FP64 peak of GB300: 152 SMs x 2 DFMA per clock x 2 flops x 2.06 GHz
 FP64_NOMINAL_GFLOPS = 1252.5
 KERNEL_SOURCES = ["emt_device.cuh", "emt_intdiv.cuh", "emt_intlog.cuh", "emt_unit.cuh", "emt_logtab.h", "emt_step.cuh",
@@ -412,7 +417,9 @@ def gpu_arm(args):
                 "mean_launch_ms": kern_ms / max(kern_launch, 1),
                 "algorithmic_flops_per_launch": flops * steps_per_launch,
                 "flops_per_track_step": flops,
-                "flops_source": "census of the oracle's step (oracle/census.py)",
+                "flops_source": "census of the oracle's step (oracle/census.py)"
+                                + ("; field substeps as the linear map" if args.workload in ("calo_field", "batched")
+                                   else ""),
                 "kernel_share_of_step": kern_ms / total_ms}
 
     # the plain form: the same events submitted and run one at a time, with

@@ -30,12 +30,14 @@ __device__ __forceinline__ uint32_t pack_tvm(int type, int vol, int model)
 // Resident threads per SM the transport kernel is compiled for (its
 // register budget), measured on GB300.
 // Field: FP64 512 (128 registers), mixed 640.  The RK4 substeps keep many
-// doubles live: at 768 threads (80 registers) their spills share the FP64
-// unit's issue queue and the field transport ran 13-14% slower.
+// doubles live: at 768 threads (80 registers) FP64 loses 1% (4,000 events in
+// 2 T: 110.7 against 109.3 ms), mixed 14% (10,000 events: 150.5 against
+// 129.7 ms).
 // No field: 768 (80 registers, a few spills).  The step is bound by the
 // latency of its dependent chain, so more warps pay: 10,000-event
 // calorimeter at 768 against 512 threads, mixed 22.12 against 22.99 ms; the
-// cylinder shells lose 0.5% in FP64 (23.38 against 23.26 ms).
+// cylinder shells lose 0.5% in FP64 (23.38 against 23.26 ms).  Later, mixed
+// at 640 / 768 / 896 / 1024: 21.60 / 20.67 / 20.65 / 21.04 ms.
 template <typename R, bool F>
 constexpr int transport_threads_per_sm()
 {
@@ -544,8 +546,8 @@ __global__ void __launch_bounds__(BS, interact_threads_per_sm<R>() / BS) k_inter
 }
 
 // Resident threads per SM of the pipelined kernel (its register budget), as
-// for the transport kernel: FP64 in a field 512 (at 768 it spills about 500
-// bytes a thread and gains nothing), otherwise 768 (80 registers).  FP64
+// for the transport kernel: FP64 in a field 512 (at 768 the 256 batched
+// events take 333 against 283 ms), otherwise 768 (80 registers).  FP64
 // calorimeter of 10,000 events at 768 against 512 threads: 46.3 against
 // 48.0 ms.
 template <typename R, bool F>

@@ -10,15 +10,15 @@
 //    step reads a dense, coalesced range per particle type and writes the
 //    survivors and secondaries compactly into the other buffer: the step
 //    is also the compaction and the particle-type partition.
-//  * Work is handed out in chunks of blockDim.x tracks of one particle type
-//    by an atomic dispenser, so every warp runs the photon or the charged
+//  * Work is handed out in chunks of up to blockDim.x tracks of one particle
+//    type (fewer when the blocks would not all get one) by an atomic dispenser, so every warp runs the photon or the charged
 //    code path only, and blocks stay busy until the step is drained.
 //  * Within a chunk the step runs in two phases.  Phase A (every lane, its
 //    own track): cross sections, step limits, propagation, continuous loss,
 //    boundary and process selection.  Tracks that interact are counting-
 //    sorted by model into shared memory; phase B runs the samplers over the
-//    sorted records, so a warp executes one model (or two, at a group
-//    boundary) instead of every model its lanes happened to select.  This
+//    sorted records, 32 of one model at a time, so a warp executes one model
+//    instead of every model its lanes happened to select.  This
 //    is the paper's one-kernel-per-model idea (Sec. 2.2) done inside one
 //    launch, without a round trip through device memory.
 //  * Output slots are reserved once per warp: a shuffle prefix sum over the
