@@ -49,7 +49,7 @@ METRIC = "track-steps/s"
 # precision and step schedule.  Reported only while the kernel sources are
 # the ones that were measured (SHA-256 below).
 TRAFFIC = {
-    "kernel_sha256": "593ae42d8a938c3cf8c71ed485a153ae10b347872d2f8252545de94fcf743838",
+    "kernel_sha256": "ef6113c0510ffbdaddedeef9c8e02aab8cb203b65e0cbf6d00a736f510c5821f",
     "bytes_per_track_step": {"calo/fp64/pipelined": 129.2, "calo/fp64/split": 122.4, "calo/mixed/pipelined": 76.7,
                              "calo/mixed/split": 86.6, "calo_field/fp64/split": 119.9,
                              "calo_field/mixed/split": 82.4},

@@ -359,9 +359,9 @@ __device__ __forceinline__ void copy_record(const InterQueue<R>& from, long long
     to.src[k] = from.src[r];
 }
 
-// The interaction phase over the n_int records of queue iq: chunks of
+// The interaction phase over the n_int records of queue iq: chunks of up to
 // kInteractRecords * BS records, each counting-sorted by model in shared
-// memory and sampled by the block's warps in sorted order.  A record whose
+// memory and sampled by the block's warps in rounds of one model.  A record whose
 // step makes two outputs needs a growth token from the `spare` slots; a
 // step without one is deferred: split schedule (kPipe false): the track is
 // copied unchanged from the input buffer qi (it repeats the whole step);

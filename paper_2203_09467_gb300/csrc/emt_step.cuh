@@ -11,18 +11,19 @@
 //    survivors and secondaries compactly into the other buffer: the step
 //    is also the compaction and the particle-type partition.
 //  * Work is handed out in chunks of up to blockDim.x tracks of one particle
-//    type (fewer when the blocks would not all get one) by an atomic dispenser, so every warp runs the photon or the charged
-//    code path only, and blocks stay busy until the step is drained.
+//    type (fewer when the blocks would not all get one) by an atomic
+//    dispenser, so every warp runs the photon or the charged code path only,
+//    and blocks stay busy until the step is drained.
 //  * Within a chunk the step runs in two phases.  Phase A (every lane, its
 //    own track): cross sections, step limits, propagation, continuous loss,
 //    boundary and process selection.  Tracks that interact are counting-
 //    sorted by model into shared memory; phase B runs the samplers over the
 //    sorted records, 32 of one model at a time, so a warp executes one model
-//    instead of every model its lanes happened to select.  This
-//    is the paper's one-kernel-per-model idea (Sec. 2.2) done inside one
-//    launch, without a round trip through device memory.
-//  * Output slots are reserved once per warp: a shuffle prefix sum over the
-//    lanes' photon and charged output counts and one atomicAdd per type.
+//    instead of every model its lanes happened to select.  This is the paper's
+//    one-kernel-per-model idea (Sec. 2.2) done inside one launch, without a
+//    round trip through device memory.
+//  * Output slots are reserved once per warp: ballots of the lanes' photon and
+//    charged outputs and one 64-bit atomic for both counts.
 //  * Capacity: a step whose outputs do not fit is discarded and the track
 //    is copied unchanged (deferred, see k_step).  A deferred track keeps its
 //    step counter, so its random stream and every result are unchanged (the
