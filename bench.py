@@ -68,7 +68,7 @@ TRAFFIC = {
 FLOPS_PER_TRACK_STEP = {"calo": 43.09, "calo_field": 243.0, "cms": 73.49, "slab": 59.05, "batched": 243.0}
 # nominal FP64 peak of GB300: 152 SMs x 2 DFMA per clock x 2 flops x 2.06 GHz
 FP64_NOMINAL_GFLOPS = 1252.5
-KERNEL_SOURCES = ["emt_device.cuh", "emt_intdiv.cuh", "emt_intlog.cuh", "emt_unit.cuh", "emt_logtab.h", "emt_step.cuh",
+KERNEL_SOURCES = ["emt_device.cuh", "emt_field.cuh", "emt_intdiv.cuh", "emt_intlog.cuh", "emt_unit.cuh", "emt_logtab.h", "emt_step.cuh",
                   "emt_split.cuh", "emt_launch.cuh", "emt_kernels_fp64.cu", "emt_kernels_fp64_persist.cu",
                   "emt_kernels_fp64_split.cu", "emt_kernels_fp64_pipe.cu", "emt_kernels_mixed.cu",
                   "emt_kernels_mixed_persist.cu", "emt_kernels_mixed_split.cu", "emt_kernels_mixed_pipe.cu"]
