@@ -182,11 +182,9 @@ bool valid_options(const emt_options& o, std::string& why)
     return true;
 }
 
-// Validate a geometry description and lay out its arrays: zb[n + 1] (plane
-// positions or shell radii) and the layer records (materials as given, see
-// mark_vacuum).  Returns an error message, or nullptr.
-const char* check_geometry(const emt_layer* layers, int n, const emt_world* w, int n_mat, int max_bins, double* zb,
-                           LayerRec* rec)
+// Validate a geometry description and lay out zb[n + 1] (plane positions or
+// shell radii).  Returns an error message, or nullptr.
+const char* check_geometry(const emt_layer* layers, int n, const emt_world* w, int n_mat, int max_bins, double* zb)
 {
     if (n < 1 || n > kMaxLayers) return "layer count out of [1, 4096]";
     if (w->n_bins < 1 || w->n_bins > max_bins) return "n_bins out of [1, max_bins]";
@@ -199,10 +197,6 @@ const char* check_geometry(const emt_layer* layers, int n, const emt_world* w, i
         if (!(layers[i].thickness_cm > 0.0)) return "layer thickness must be positive";
         if (layers[i].material < -1 || layers[i].material >= n_mat) return "layer material index";
         zb[i + 1] = zb[i] + layers[i].thickness_cm;
-        rec[i] = LayerRec{{zb[i], zb[i + 1]},
-                          layers[i].material,
-                          layers[i].score_bin,
-                          {ord_key(zb[i] + kChordMargin), ord_key(zb[i + 1] - kChordMargin)}};
     }
     if (w->geometry == EMT_GEOM_LAYERS) {
         if (!(w->half_x_cm > 0.0) || !(w->half_y_cm > 0.0)) return "stack half widths";
@@ -218,6 +212,16 @@ const char* check_geometry(const emt_layer* layers, int n, const emt_world* w, i
     if (b2 > 0.0 && (!(w->rk_delta_cm > 0.0) || !(w->max_field_step_cm > 0.0)))
         return "field needs rk_delta_cm > 0 and max_field_step_cm > 0";
     return nullptr;
+}
+
+// records of n layers (materials as given, see mark_vacuum) between the planes z[0..n]
+void layer_records(const emt_layer* layers, const double* z, int n, LayerRec* rec)
+{
+    for (int i = 0; i < n; ++i)
+        rec[i] = LayerRec{{z[i], z[i + 1]},
+                          layers[i].material,
+                          layers[i].score_bin,
+                          {ord_key(z[i] + kChordMargin), ord_key(z[i + 1] - kChordMargin)}};
 }
 
 // the step kernels' material index of a layer: -1 for a vacuum material
@@ -1231,8 +1235,9 @@ emt_status emt_load_geometry(emt_ctx* c, const emt_layer* layers, int32_t n, con
     if (n < 1 || n > kMaxLayers) return fail(c, EMT_ERR_INVALID_ARG, "layer count out of [1, 4096]");
     std::vector<double> zb(n + 1);
     std::vector<LayerRec> rec(n);
-    if (const char* why = check_geometry(layers, n, w, c->n_mat, c->opt.max_bins, zb.data(), rec.data()))
+    if (const char* why = check_geometry(layers, n, w, c->n_mat, c->opt.max_bins, zb.data()))
         return fail(c, EMT_ERR_INVALID_ARG, why);
+    layer_records(layers, zb.data(), n, rec.data());
     if (cudaSetDevice(c->opt.device) != cudaSuccess) return fail(c, EMT_ERR_CUDA, "cudaSetDevice");
     const Plan& pl = c->plan;
     EMT_CUDA(c, cudaMemcpyAsync(c->pool + pl.zb, zb.data(), sizeof(double) * (n + 1), cudaMemcpyHostToDevice, c->stream));
@@ -1777,12 +1782,23 @@ extern "C" emt_status emt_transport_static(int32_t device, uint32_t seed, const 
 
     // ---- geometry
     double zb[kMaxLayers + 1];
-    LayerRec rec[kMaxLayers];
-    if (check_geometry(layers, n_layers, w, n_mat, EMT_STATIC_MAX_BINS, zb, rec)) return EMT_ERR_INVALID_ARG;
-    mark_vacuum(rec, n_layers, vac);
-    if (cudaMemcpyAsync(pool + pl.zb, zb, sizeof(double) * (n_layers + 1), cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(pool + pl.layer, rec, sizeof(LayerRec) * n_layers, cudaMemcpyHostToDevice, st) != cudaSuccess)
+    if (check_geometry(layers, n_layers, w, n_mat, EMT_STATIC_MAX_BINS, zb)) return EMT_ERR_INVALID_ARG;
+    if (cudaMemcpyAsync(pool + pl.zb, zb, sizeof(double) * (n_layers + 1), cudaMemcpyHostToDevice, st) != cudaSuccess)
         return EMT_ERR_CUDA;
+    // The records go up through a small buffer, since the caller's thread may
+    // have little stack (all 4,096 would take 128 KB of it).  A full buffer is
+    // waited for before it is filled again.
+    constexpr int kLayersAtOnce = 512;
+    LayerRec rec[kLayersAtOnce];
+    for (int i = 0; i < n_layers; i += kLayersAtOnce) {
+        const int m = std::min(n_layers - i, kLayersAtOnce);
+        if (i > 0 && cudaStreamSynchronize(st) != cudaSuccess) return EMT_ERR_CUDA;
+        layer_records(layers + i, zb + i, m, rec);
+        mark_vacuum(rec, m, vac);
+        if (cudaMemcpyAsync(pool + pl.layer + sizeof(LayerRec) * i, rec, sizeof(LayerRec) * m, cudaMemcpyHostToDevice,
+                            st) != cudaSuccess)
+            return EMT_ERR_CUDA;
+    }
     set_geometry(p, n_layers, w, zb);
 
     // ---- events: slots 0..n_events-1 in order; primaries read in place
