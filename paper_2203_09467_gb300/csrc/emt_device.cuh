@@ -969,7 +969,7 @@ struct FieldStages {
     float kq, hs, h6;
 };
 
-__device__ __forceinline__ FieldStages field_step(const Params<float>& p, double kq, double h, const float*, bool)
+__device__ __forceinline__ FieldStages field_step(const Params<float>& p, double kq, double h, const float*, int)
 {
     (void)p;
     FieldStages f;
@@ -1108,7 +1108,7 @@ __device__ __forceinline__ double propagate_field(const Params<R>& p, int charge
     const double kq = mdiv(charge < 0 ? -kFieldC : kFieldC, pm);
     double s = 0.0;
     *crossed = false;
-    const auto whole = field_step(p, kq, hs, u, n > 1);
+    const auto whole = field_step(p, kq, hs, u, n);
     double x1[3];
     R u1[3];
     for (int i = 0; i < n;) {
@@ -1131,7 +1131,7 @@ __device__ __forceinline__ double propagate_field(const Params<R>& p, int charge
         Exit e;
         if (chord_exit<G>(p, vol, x, x1, e)) {
             h = __dmul_rn(hs, e.t);
-            rk4(p, field_step(p, kq, h, u, false), h, x, u, x1, u1);
+            rk4(p, field_step(p, kq, h, u, 1), h, x, u, x1, u1);
             *evals += 1;
             snap(e, x1);
             *bnd = e;

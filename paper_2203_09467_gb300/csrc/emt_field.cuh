@@ -34,9 +34,9 @@ namespace emt {
 //
 // Over n substeps c is not quite constant (|w1|^2 gains g - e of itself in
 // each) and the axis component grows by (1 + c)^n: what this leaves out of the
-// direction is of the size n^2 e g / 4.  For |g| < 2^-34, a turn t below 0.040,
-// and the at most 100 substeps of a step that is below 2^-56 (the default miss
-// distance and cut give t < 0.02 in 2 T).  Larger turns, and a u that does not
+// direction is of the size n^2 e g / 4, below 2^-54 for n |g| < 2^-26: turns t
+// below 0.045 at 100 substeps, 0.07 at 8 (the default miss distance and cut
+// give t < 0.02 in 2 T).  Larger turns, and a u that does not
 // have unit length to start with, are renormalised after each substep; there
 // the rounding of t and of the coefficients, the same in every substep, would
 // be a phase error that grows with n, so the two turning coefficients are
@@ -60,10 +60,21 @@ struct FieldMap {
     bool renormalise;  // after every substep
 };
 
-// more: other substeps follow this map's (after the last one field_end takes
-// care of the length)
+// whether n |g| < 2^-26, with n > 1 rounded up to a power of two (exponent
+// arithmetic: no instruction on the FP64 pipe)
+EMT_FLD bool constant_loss(double g, int n)
+{
+#if defined(__CUDA_ARCH__)
+    const int log2_n = 32 - __clz(n - 1);
+#else
+    const int log2_n = 32 - __builtin_clz((unsigned)(n - 1));
+#endif
+    return ((int)(intdiv::dbits(g) >> 32) & 0x7FFFFFFF) + (log2_n << 20) < ((1023 - 26) << 20);
+}
+
+// n: substeps of this length (after the last one field_end takes care of the length)
 template <typename P>
-EMT_FLD FieldMap field_step(const P& p, double kq, double h, const double* u, bool more)
+EMT_FLD FieldMap field_step(const P& p, double kq, double h, const double* u, int n)
 {
     FieldMap f;
     const double b = p.baxis >= 0 ? p.B[p.baxis] : p.bmag;
@@ -80,7 +91,7 @@ EMT_FLD FieldMap field_step(const P& p, double kq, double h, const double* u, bo
     f.c = 0.0;
     f.sa = 0.0;
     f.renormalise = false;
-    if (more) {
+    if (n > 1) {
         // w = -|w1|^2 / 2 with |w1|^2 = |u|^2 - (u b)^2; g = g_tt t^2
         const double uu = fma(u[0], u[0], fma(u[1], u[1], u[2] * u[2]));
         const double ub =
@@ -88,7 +99,7 @@ EMT_FLD FieldMap field_step(const P& p, double kq, double h, const double* u, bo
         const double w = -0.5 * fma(-ub, ub, uu);
         const double g_tt = tt * tt * fma(tt, 1.0 / 576.0, -1.0 / 72.0);
         const double g = g_tt * tt;
-        f.renormalise = !(fabs(g) < 0x1p-34 && fabs(uu - 1.0) < 0x1p-48);
+        f.renormalise = !(constant_loss(g, n) && fabs(uu - 1.0) < 0x1p-48);
         if (!f.renormalise) {
             f.c = w * g;
             f.sa = w * g_tt * (t * k) * ub;

@@ -113,7 +113,7 @@ int main(int argc, char** argv)
                     double xm[3] = {0, 0, 0}, um[3] = {u[0], u[1], u[2]}, xs[3] = {0, 0, 0}, us[3] = {u[0], u[1], u[2]};
                     quad xq[3] = {0, 0, 0}, uq[3] = {u[0], u[1], u[2]};
                     const quad Bq[3] = {f.B[0], f.B[1], f.B[2]};
-                    const emt::FieldMap map = emt::field_step(f, kq, h, um, n > 1);
+                    const emt::FieldMap map = emt::field_step(f, kq, h, um, n);
                     double s = 0.0;
                     for (int i = 0; i < n; ++i) {
                         double xo[3], uo[3];
