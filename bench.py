@@ -49,10 +49,10 @@ METRIC = "track-steps/s"
 # precision and step schedule.  Reported only while the kernel sources are
 # the ones that were measured (SHA-256 below).
 TRAFFIC = {
-    "kernel_sha256": "ef6113c0510ffbdaddedeef9c8e02aab8cb203b65e0cbf6d00a736f510c5821f",
-    "bytes_per_track_step": {"calo/fp64/pipelined": 129.2, "calo/fp64/split": 122.4, "calo/mixed/pipelined": 76.7,
-                             "calo/mixed/split": 86.6, "calo_field/fp64/split": 119.9,
-                             "calo_field/mixed/split": 82.4},
+    "kernel_sha256": "11757a7448d5441f2cb5d750f8892700a153aeef62a0d58232ffe50ecb015d58",
+    "bytes_per_track_step": {"calo/fp64/pipelined": 129.4, "calo/fp64/split": 122.4, "calo/mixed/pipelined": 76.6,
+                             "calo/mixed/split": 86.6, "calo_field/fp64/split": 120.0,
+                             "calo_field/mixed/split": 82.5},
     "source": "profiles/step_kernels_dram_traffic.md",
 }
 # Algorithmic FP64 work of one track-step of the method, fixed by its
@@ -62,14 +62,14 @@ TRAFFIC = {
 # (comparisons and elementary functions are listed there, not counted).  It
 # does not change when the kernels are optimised, except that the field
 # workloads count what a step needs once the RK4 stages of a uniform field are
-# collapsed to a linear map (emt_device.cuh): 23 flops per substep along an
+# collapsed to a linear map (emt_field.cuh): 23 flops per substep along an
 # axis, 7.16 substeps per track-step, 35 flops for the map, and the 43.1 of a
 # step without a field (stage by stage the census counts 968).
 FLOPS_PER_TRACK_STEP = {"calo": 43.09, "calo_field": 243.0, "cms": 73.49, "slab": 59.05, "batched": 243.0}
 # nominal FP64 peak of GB300: 152 SMs x 2 DFMA per clock x 2 flops x 2.06 GHz
 FP64_NOMINAL_GFLOPS = 1252.5
-KERNEL_SOURCES = ["emt_device.cuh", "emt_field.cuh", "emt_intdiv.cuh", "emt_intlog.cuh", "emt_unit.cuh", "emt_logtab.h", "emt_step.cuh",
-                  "emt_split.cuh", "emt_launch.cuh", "emt_kernels_fp64.cu", "emt_kernels_fp64_persist.cu",
+KERNEL_SOURCES = ["emt_device.cuh", "emt_field.cuh", "emt_intdiv.cuh", "emt_intlog.cuh", "emt_unit.cuh",
+                  "emt_logtab.h", "emt_step.cuh", "emt_split.cuh", "emt_launch.cuh", "emt_kernels_fp64.cu", "emt_kernels_fp64_persist.cu",
                   "emt_kernels_fp64_split.cu", "emt_kernels_fp64_pipe.cu", "emt_kernels_mixed.cu",
                   "emt_kernels_mixed_persist.cu", "emt_kernels_mixed_split.cu", "emt_kernels_mixed_pipe.cu"]
 

@@ -308,7 +308,7 @@ struct emt_ctx {
     // resident blocks of the step kernels without and with a field
     int resident_blocks[2] = {0, 0};  // fused schedule
     int resident_a[2] = {0, 0};       // split schedule: transport kernel
-    int resident_b = 0;               // split schedule: interaction kernel
+    int resident_b = 0;               // split schedule: interaction kernel; grid of the sorting launches
     int resident_p[2] = {0, 0};       // pipelined schedule
     int persist_grid[2] = {0, 0};     // persistent step loop (cooperative launch)
     long long wait_cycles = 0;           // bound of one grid-barrier wait, SM clock cycles
@@ -1069,7 +1069,7 @@ emt_status emt_create(const emt_options* o, emt_ctx** out)
     for (int f = 0; f < 2; ++f) {
         const bool field = f != 0;
         const int bs = c->block;
-        // only the kernels that this context can launch are asked for
+        // of the step kernels, only those that this context can launch are asked for
         if (!c->plan.split)
             c->resident_blocks[f] = resident([&] { return Launch<float>::max_blocks_per_sm(bs, field); },
                                              [&] { return Launch<double>::max_blocks_per_sm(bs, field); });
@@ -1080,6 +1080,9 @@ emt_status emt_create(const emt_options* o, emt_ctx** out)
             c->resident_p[f] = resident([&] { return Launch<float>::max_blocks_pipe(bs, field); },
                                         [&] { return Launch<double>::max_blocks_pipe(bs, field); });
     }
+    // interaction kernel; also the grid of the two sorting launches in a field
+    // (256 threads, few registers: any grid that fills the SMs will do), which
+    // is all that the pipelined schedule uses it for
     if (c->plan.split)
         c->resident_b = resident([&] { return Launch<float>::max_blocks_interact(c->block, select); },
                                  [&] { return Launch<double>::max_blocks_interact(c->block, select); });

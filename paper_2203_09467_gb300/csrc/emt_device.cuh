@@ -7,7 +7,9 @@
 // float for the mixed path (positions, boundary distances and tallies stay
 // FP64).  Each formula cites the textbook closed form it evaluates; the
 // operation order of the FP64 instantiation is the library's definition of
-// the method and is what the FP64 tests compare against.
+// the method and is what the FP64 tests compare against, except for the
+// substeps in a field: the same RK4 as a linear map, with roundings of its own
+// (emt_field.cuh).
 #pragma once
 
 #include <cstdint>
@@ -237,8 +239,8 @@ struct InterQueue {
 // Four values read together: what a lookup needs of a table node lies in
 // one aligned record (one 16-byte load in float, two in FP64), so that a
 // lookup waits for memory once instead of once per table.  With the layer
-// records below: calorimeter of 10,000 events, mixed 21.6 -> 20.8 ms, FP64
-// 38.1 -> 37.8 ms; in 2 T, 4,000 events FP64, 142 -> 139 ms.
+// records below, and the kernels otherwise as they were then: calorimeter of
+// 10,000 events 3.4% faster in mixed precision and 1% in FP64, in 2 T FP64 2.3%.
 template <typename R>
 struct alignas(4 * sizeof(R)) Quad {
     R a, b, c, d;
@@ -896,10 +898,10 @@ __device__ __forceinline__ Exit nav_exit(const Params<R>& p, int vol, const doub
 // stage, positions in FP64.  A: the axis of a field along one coordinate
 // axis (-1: any direction).  Along an axis the products with B's zero
 // components are zeros and the component of u along B does not change, so
-// leaving them out changes no result (45 instead of 72 operations):
-// calorimeter in 2 T, 10,000 events, 252.7 -> 203.7 ms (with the chord test
-// below on the integer pipe), and 201.0 -> 162.6 ms with its 32-bit keys and
-// the division by a length near 1 (emt_unit.cuh).
+// leaving them out changes no result (45 instead of 72 operations): the
+// calorimeter in 2 T (10,000 events, 130 ms) ran 1.24 times as fast with it and
+// the chord test below on the integer pipe, and 1.24 times again with that
+// test's 32-bit keys and the division by a length near 1 (emt_unit.cuh).
 template <int A>
 __device__ __forceinline__ void rk4_stages(const Params<float>& p, float kq, const double x[3], const float u[3],
                                            float hs, float h6, double xo[3], float uo[3])
@@ -1048,7 +1050,12 @@ __device__ __forceinline__ bool chord_inside(const Params<R>& p, int vol, const 
     }
     // Layers: 32-bit integer comparisons through ord_key with the bounds' keys
     // formed when the geometry is loaded (true only when the exact comparisons
-    // are).  A NaN coordinate of x1 fails one of the tests of its axis.
+    // are).  A NaN coordinate of x1 fails one of the tests of its axis.  The
+    // keys resolve 1e-6 of a coordinate (2^-20): in a layer thinner than about
+    // 2e-6 of its distance from the origin the test never passes and every
+    // substep pays chord_exit's quotient, with the same results.  Substeps are
+    // mostly longer than such a layer unless it lies tens of metres away, so
+    // nearly every one of them crosses a plane there in any case.
     if (vol >= 0) {
         const int k2 = ord_key(x1[2]);
         const LayerRec& l = p.layer[vol];
@@ -1097,9 +1104,10 @@ __device__ __forceinline__ bool chord_exit(const Params<R>& p, int vol, const do
 // out together (worked out where they fall, each ran the navigation for a
 // lane or two).  With the quotient of chord_exit and the conversions and
 // comparisons off the FP64 pipe: calorimeter in 2 T, FP64 4,000 events
-// 138.9 -> 109.7 ms, mixed 10,000 events 163.2 -> 129.9 ms; a served stream of
-// small populations loses 2% (84.5 -> 86.4 ms) to the longer dependent chain
-// of a substep.  Returns the path length; *evals counts the integrator
+// 138.9 -> 109.7 ms, mixed 10,000 events 163.2 -> 129.9 ms (109.5 and 130.0 with
+// the present kernels); a served stream of small populations lost 2% to the
+// longer dependent chain of a substep (84.5 -> 86.4 ms, now 86.6).  Returns the
+// path length; *evals counts the integrator
 // evaluations.
 template <int G, typename R>
 __device__ __forceinline__ double propagate_field(const Params<R>& p, int charge, double pm, int vol, double x[3],

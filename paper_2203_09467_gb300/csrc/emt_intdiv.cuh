@@ -40,7 +40,8 @@
 //
 // 32-bit words in the first Newton step and one-sided errors (one
 // correction instead of two) in place of 128-bit products throughout:
-// 10,000-event calorimeter in FP64 46.5 -> 42.8 ms, one event 4.28 -> 4.01 ms.
+// 10,000-event calorimeter in FP64 46.5 -> 42.8 ms, one event 4.28 -> 4.01 ms
+// (36.8 and 3.20 ms with everything else the kernels have changed since).
 //
 // The FP32 reciprocal (square root) estimates are the only floating-point
 // steps; their exact values do not matter, only their error bounds.  Host

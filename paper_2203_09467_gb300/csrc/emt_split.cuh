@@ -6,8 +6,12 @@
 // a barrier while a few run the samplers.  Here the transport kernel runs
 // phase A for every track and appends the tracks that interact to a global
 // queue (warp-aggregated, one atomic per warp); the interaction kernel then
-// takes the queue in full chunks, counting-sorts each chunk by model in
-// shared memory and samples with every lane busy.  The cost is one more
+// takes the queue in chunks (of up to kInteractRecords records per thread,
+// smaller for a short queue), counting-sorts each chunk by model in shared
+// memory and samples it in rounds of up to 32 records of one model, which the
+// block's warps take from a shared counter.  The last round of each model is
+// partly filled and rejection loops end at different trips: 17 to 19 of 32
+// lanes are active on average.  The cost is one more
 // write and read of the interacting tracks' state (a few percent of the
 // step's track-state traffic); the results are the same as the fused
 // schedule's (same arithmetic, same random streams).
@@ -27,17 +31,20 @@ __device__ __forceinline__ uint32_t pack_tvm(int type, int vol, int model)
 // the same random numbers when they do step and no result depends on the
 // policy; both kernels count their outputs' energy classes for the next
 // step's selection.
+//
 // Resident threads per SM the transport kernel is compiled for (its
-// register budget), measured on GB300.
-// Field: FP64 512 (128 registers), mixed 640.  The RK4 substeps keep many
-// doubles live: at 768 threads (80 registers) FP64 loses 1% (4,000 events in
-// 2 T: 110.7 against 109.3 ms), mixed 14% (10,000 events: 150.5 against
-// 129.7 ms).
+// register budget), measured on GB300.  The launch bound is this over the
+// block size in whole blocks: 640 is 5 blocks of 128, but 2 of 256 (512
+// threads, 128 registers).
+// Field: FP64 512 (128 registers), mixed 640.  The substeps keep many
+// doubles live: at 768 threads (80 registers, blocks of 256) FP64 loses 1%
+// (4,000 events in 2 T: 110.8 against 109.5 ms), mixed 14% (10,000 events:
+// 150.8 against 130.0 ms), a served stream 6% (92.5 against 86.6 ms).
 // No field: 768 (80 registers, a few spills).  The step is bound by the
-// latency of its dependent chain, so more warps pay: 10,000-event
-// calorimeter at 768 against 512 threads, mixed 22.12 against 22.99 ms; the
-// cylinder shells lose 0.5% in FP64 (23.38 against 23.26 ms).  Later, mixed
-// at 640 / 768 / 896 / 1024: 21.60 / 20.67 / 20.65 / 21.04 ms.
+// latency of its dependent chain, so more warps pay: 10,000-event calorimeter
+// in mixed precision (blocks of 128) 20.3 against 22.7 ms at 512; FP64 shells
+// and the run with every option are level.  640 was 4% slower, 896 no better,
+// 1024 2% slower.
 template <typename R, bool F>
 constexpr int transport_threads_per_sm()
 {
@@ -324,9 +331,10 @@ __global__ void __launch_bounds__(BS, transport_threads_per_sm<R, F>() / BS)
 // counting-sorts kInteractRecords * BS records by model and its warps take
 // rounds of 32 records of one model from a shared counter.  Larger chunks have
 // fewer partly filled rounds; rounds taken as warps come free even out models
-// of different cost.  4 against 2 with fixed rounds: cylinder shells 20.9 ->
-// 20.1 ms, every option on 37.1 -> 36.5 ms, FP64 calorimeter 37.5 -> 37.1 ms,
-// mixed unchanged; 8 gives the shells nothing.
+// of different cost.  4 against 2: 256 batched events in FP64 279 against
+// 325 ms, cylinder shells 20.1 against 20.5, calorimeter FP64 36.8 against 37.2
+// and mixed 20.3 against 20.4, every option on level; 8 gives the shells
+// nothing.
 constexpr int kInteractRecords = 4;
 
 // Records in one chunk of an interaction phase over n records on `grid`
@@ -511,9 +519,9 @@ __device__ __forceinline__ void interact_chunks(const Params<R>& p, const Tracks
 }
 
 // Resident threads per SM of the interaction kernel (its register budget):
-// FP64 512 (at 768 the shells lose 3.2% and the run with every option 7%),
-// mixed 768 (against 512: calorimeter of 10,000 events 21.8 -> 21.6 ms, in 2 T
-// 203.8 -> 201.1 ms).
+// FP64 512 (at 768 the shells take 20.9 instead of 20.1 ms, the run with every
+// option 39.2 instead of 36.5), mixed 768 (at 512 the calorimeter of 10,000
+// events takes 20.5 instead of 20.3 ms, in 2 T 132.0 instead of 130.0).
 template <typename R>
 constexpr int interact_threads_per_sm()
 {
@@ -547,9 +555,8 @@ __global__ void __launch_bounds__(BS, interact_threads_per_sm<R>() / BS) k_inter
 
 // Resident threads per SM of the pipelined kernel (its register budget), as
 // for the transport kernel: FP64 in a field 512 (at 768 the 256 batched
-// events take 333 against 283 ms), otherwise 768 (80 registers).  FP64
-// calorimeter of 10,000 events at 768 against 512 threads: 46.3 against
-// 48.0 ms.
+// events take 331 against 279 ms), otherwise 768 (80 registers; FP64
+// calorimeter of 10,000 events 36.8 ms, 36.9 at 512).
 template <typename R, bool F>
 constexpr int pipe_threads_per_sm()
 {

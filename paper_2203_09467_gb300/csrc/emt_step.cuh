@@ -716,9 +716,10 @@ struct Staging {
 // samplers one after the other; with a round of its own each model of a
 // small chunk is sampled by another warp at the same time.  Every warp forms
 // the groups from the shared counts on its own (lane m holds model m).  With
-// chunks that shrink to the population (below, and interact_chunk): one
-// 10 GeV event 4.09 -> 3.33 ms, 1,000 x 100 MeV into the slab 1.22 -> 0.99 ms,
-// FP64 calorimeter of 10,000 events 43.0 -> 39.4 ms, mixed 22.2 ms as before.
+// chunks that shrink to the population (below, and interact_chunk), and the
+// kernels otherwise as they were then: one 10 GeV event 4.09 -> 3.33 ms (now
+// 3.20), 1,000 x 100 MeV into the slab 1.22 -> 0.99 ms (0.96), FP64 calorimeter
+// of 10,000 events 43.0 -> 39.4 ms (36.8), mixed level.
 struct ModelGroups {
     int count, first;          // records of the lane's model, records before it
     int rounds_end;            // rounds up to and including the lane's model
@@ -920,6 +921,12 @@ __device__ __forceinline__ void step_body(const Params<R>& p, int side, int cin,
     flush_tally<F>(p, lane, tally);
 }
 
+// 512 resident threads per SM (128 registers) with and without a field, here
+// and in k_persist: at 768 without a field one 10 GeV event takes 3.39 instead
+// of 3.20 ms, 37 events 8.20 instead of 7.79, the slab 1.00 instead of 0.96 (few
+// warps, whose spills lengthen the chain of a step).  10,000 events gain from 768
+// (FP64 76.2 -> 73.2 ms, mixed 31.7 -> 28.9), but take 37 and 20 ms in the other
+// schedules.
 template <typename R, int BS, int G, bool F, bool X>
 __global__ void __launch_bounds__(BS, 512 / BS) k_step(Params<R> p, int side, int cin, int cout, int cclr)
 {
